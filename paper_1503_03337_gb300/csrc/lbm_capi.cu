@@ -1,5 +1,6 @@
 // C-ABI of liblbm: handle lifecycle, parameter validation and the host
 // orchestration of the single-domain kernels (declared in include/lbm.h).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -388,10 +389,14 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   DeviceGuard dg(h->device);
   const int K = h->params.residual_interval;
   const bool neq = (h->d.neq_vel | h->d.neq_pre) != 0;
-  for (int64_t k = 0; k < nsteps; ++k) {
-    cudaError_t e = launch_step(h->d, h->n, h->block, h->stream);
+  while (nsteps > 0) {
+    // up to the next boundary pass or reduction
+    int64_t m = neq ? 1 : nsteps;
+    if (K > 0) m = std::min<int64_t>(m, K - h->n % K);
+    cudaError_t e = launch_steps(h->d, h->n, m, h->block, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
-    h->n += 1;
+    h->n += m;
+    nsteps -= m;
     if (neq) {  // the extrapolation boundaries of the new time level
       e = launch_neq(h->d, h->n, h->stream);
       if (e != cudaSuccess) return cuda_fail(e, "boundary kernel");
@@ -614,9 +619,10 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
                        (int64_t)h->d.Q * h->d.N >= (int64_t(1) << 31)))
       continue;
     int64_t n = n0;
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = launch_step(h->d, n++, b, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, h->stream);
+    n += 2;
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    for (int k = 0; k < trials && e == cudaSuccess; ++k) e = launch_step(h->d, n++, b, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, trials, b, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float t = 0.f;

@@ -68,8 +68,9 @@ void set_last_error(const std::string& msg);
 // F(t_n) of a domain.
 void force_at(const DomainDesc& d, int64_t n, double F[3]);
 
-// Queue one fused step n -> n+1 (parity n & 1).
-cudaError_t launch_step(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st);
+// Queue the fused steps n .. n + count - 1 (parity of each its number's).
+cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                         cudaStream_t st);
 
 // f = f_eq(p - p_ref, u) at every node, stored for step 0 (even layout).
 cudaError_t launch_init(const DomainDesc& d, const double* u, const double* p,

@@ -563,13 +563,18 @@ __host__ __device__ inline void scale_rows(Rates<R>& r) {
     r.h[K] = R(0);
     r.g[K] = R(0);
   }
-  for (int K = 0; K < Q; ++K) {
-    const R inv = R(1.0 / row_norm<Q>(K));
-    const R sk = rate_of<Q>(r, K);
-    r.k[K] = sk * inv;
-    r.h[K] = (K == 2 || K == 4 || K == 6) ? inv : (R(1) - R(0.5) * sk) * inv;
-    r.g[K] = (R(1) - sk) * inv;
-  }
+  [&]<int... K>(std::integer_sequence<int, K...>) {
+    (
+        [&] {
+          constexpr double norm = row_norm<Q>(K);
+          const R inv = R(1.0 / norm);
+          const R sk = rate_of<Q>(r, K);
+          r.k[K] = sk * inv;
+          r.h[K] = (K == 2 || K == 4 || K == 6) ? inv : (R(1) - R(0.5) * sk) * inv;
+          r.g[K] = (R(1) - sk) * inv;
+        }(),
+        ...);
+  }(std::make_integer_sequence<int, Q>{});
 }
 
 // ---------------------------------------------------------------------------

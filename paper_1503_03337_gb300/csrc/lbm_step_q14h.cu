@@ -4,11 +4,13 @@
 
 namespace lbm {
 
-cudaError_t launch_step_q14_bf16(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st);
+cudaError_t launch_step_q14_bf16(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                                 cudaStream_t st);
 
-cudaError_t launch_step_q14_half(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st) {
-  if (d.storage == LBM_STORAGE_F16) return launch_typed<14, __half, float>(d, n, b, st);
-  return launch_step_q14_bf16(d, n, b, st);
+cudaError_t launch_step_q14_half(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                                 cudaStream_t st) {
+  if (d.storage == LBM_STORAGE_F16) return launch_typed<14, __half, float>(d, n, count, b, st);
+  return launch_step_q14_bf16(d, n, count, b, st);
 }
 
 }  // namespace lbm

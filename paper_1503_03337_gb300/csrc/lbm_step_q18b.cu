@@ -3,8 +3,9 @@
 
 namespace lbm {
 
-cudaError_t launch_step_q18_bf16(const DomainDesc& d, int64_t n, BlockShape b, cudaStream_t st) {
-  return launch_typed<18, __nv_bfloat16, float>(d, n, b, st);
+cudaError_t launch_step_q18_bf16(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                                 cudaStream_t st) {
+  return launch_typed<18, __nv_bfloat16, float>(d, n, count, b, st);
 }
 
 }  // namespace lbm
