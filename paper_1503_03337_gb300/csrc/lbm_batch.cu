@@ -373,6 +373,20 @@ int grid_for_batch(lbm_batch* b) {
   return per_sm * sms;
 }
 
+// Step s (of the chunk) of planes z0 .. z0 + planes - 1 of solo entry k.
+cudaError_t launch_solo_step(lbm_batch* b, const lbm_batch::Group& g, int k, int s, int z0,
+                             int planes, dim3 block) {
+  const BatchEntry& he = b->host_ents[k];
+  const int periodic = he.period > 0.0;
+  SoloLaunch sl{g.storage, g.sr, g.force, (g.parity + s) & 1, periodic,
+                dim3(he.tiles_x, he.tiles_y, planes), block, b->stream, he.d,
+                b->dyn + (size_t)(s % kDynSteps) * b->capacity + k};
+  sl.d.z0 = z0;
+  if (!periodic)  // constant force in the descriptor
+    for (int a = 0; a < 3; ++a) sl.d.F[a] = float(he.force[a]);
+  return g.Q == 14 ? launch_solo_q14(sl) : launch_solo_q18(sl);
+}
+
 // Step s (of the chunk) of one group: one launch per solo entry, or one
 // grouped launch.
 cudaError_t launch_group_step(lbm_batch* b, const lbm_batch::Group& g, int s,
@@ -380,16 +394,8 @@ cudaError_t launch_group_step(lbm_batch* b, const lbm_batch::Group& g, int s,
   const StepDyn* dyn = b->dyn + (size_t)(s % kDynSteps) * b->capacity;
   const bool odd = ((g.parity + s) & 1) != 0;
   if (g.solo) {
-    for (int k = g.first; k < g.first + g.count; ++k) {
-      const BatchEntry& he = b->host_ents[k];
-      const int periodic = he.period > 0.0;
-      SoloLaunch sl{g.storage, g.sr, g.force, odd ? 1 : 0, periodic,
-                    dim3(he.tiles_x, he.tiles_y, he.d.nz), block, b->stream, he.d, dyn + k};
-      if (!periodic)  // constant force in the descriptor
-        for (int a = 0; a < 3; ++a) sl.d.F[a] = float(he.force[a]);
-      cudaError_t e = g.Q == 14 ? launch_solo_q14(sl) : launch_solo_q18(sl);
-      if (e != cudaSuccess) return e;
-    }
+    for (int k = g.first; k < g.first + g.count; ++k)
+      if (cudaError_t e = launch_solo_step(b, g, k, s, 0, b->host_ents[k].d.nz, block)) return e;
     return cudaSuccess;
   }
   // contiguous runs of tiles per CTA, short enough to leave about eight
@@ -429,6 +435,18 @@ cudaError_t enqueue_chunk(lbm_batch* b, int chunk) {
       while (g0 < b->groups.size()) {  // one cluster: groups g0 .. g1-1
         size_t g1 = g0;
         while (g1 < b->groups.size() && b->groups[g1].cluster == b->groups[g0].cluster) ++g1;
+        const lbm_batch::Group& g = b->groups[g0];
+        if (g1 == g0 + 1 && g.solo && g.count == 1) {  // alone in L2: slab by slab
+          const DomainDesc& dd = b->slots[b->order[g.first]].dd;
+          cudaError_t e = run_slabs(dd.nz, dd.per[2] != 0, slab_plan(dd, b->l2_bytes), ns,
+                                    [&](int64_t s, int z0, int planes) {
+                                      return launch_solo_step(b, g, g.first, s0 + (int)s, z0,
+                                                              planes, block);
+                                    });
+          if (e != cudaSuccess) return e;
+          g0 = g1;
+          continue;
+        }
         for (int s = s0; s < s0 + ns; ++s)
           for (size_t gi = g0; gi < g1; ++gi)
             if (cudaError_t e = launch_group_step(b, b->groups[gi], s, local, block))

@@ -34,6 +34,7 @@ struct lbm_handle {
   void* staging = nullptr;      // grow-only device buffer for host transfers
   size_t staging_bytes = 0;
   int64_t bytes = 0;
+  int64_t l2_bytes = 0;         // the device's L2 size
   uint8_t* solid_bytes = nullptr;   // N bytes: the solid-node mask, or null
   uint32_t* solid_links = nullptr;  // N words: its link bits (d.solid)
 };
@@ -178,6 +179,10 @@ int lbm_create(const lbm_desc* desc, void* cuda_stream, lbm_handle** out) {
     delete h;
     return cuda_fail(e, "cudaGetDevice");
   }
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device) == cudaSuccess)
+    h->l2_bytes = l2;
+  else cudaGetLastError();
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   h->d.Q = desc->Q;
   h->d.nx = desc->nx;
@@ -389,11 +394,12 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   DeviceGuard dg(h->device);
   const int K = h->params.residual_interval;
   const bool neq = (h->d.neq_vel | h->d.neq_pre) != 0;
+  const SlabPlan plan = slab_plan(h->d, h->l2_bytes);
   while (nsteps > 0) {
     // up to the next boundary pass or reduction
     int64_t m = neq ? 1 : nsteps;
     if (K > 0) m = std::min<int64_t>(m, K - h->n % K);
-    cudaError_t e = launch_steps(h->d, h->n, m, h->block, h->stream);
+    cudaError_t e = launch_steps(h->d, h->n, m, h->block, plan, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
     h->n += m;
     nsteps -= m;
@@ -610,6 +616,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
   BlockShape best = h->block;
   double best_ms = 1e300;
   const int64_t n0 = h->n;
+  const SlabPlan plan = slab_plan(h->d, h->l2_bytes);
   const int xmax = ((h->d.nx + 31) / 32) * 32;
   for (BlockShape b : kCandidates) {
     if (e != cudaSuccess) break;
@@ -619,10 +626,10 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
                        (int64_t)h->d.Q * h->d.N >= (int64_t(1) << 31)))
       continue;
     int64_t n = n0;
-    if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, plan, h->stream);
     n += 2;
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    if (e == cudaSuccess) e = launch_steps(h->d, n, trials, b, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, trials, b, plan, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float t = 0.f;

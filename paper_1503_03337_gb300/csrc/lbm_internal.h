@@ -68,9 +68,55 @@ void set_last_error(const std::string& msg);
 // F(t_n) of a domain.
 void force_at(const DomainDesc& d, int64_t n, double F[3]);
 
+// Slabs of planes that run several steps each while their populations stay
+// in L2 (slabs = 1: every step sweeps the whole box).  Neighbouring planes may
+// be one step apart and no more, so a slab moves down one plane per step:
+//   slab k runs step s of a round on planes [begin(k) - s, begin(k + 1) - s),
+// the first one from plane 0 on and the last one up to the top, and slab k
+// finishes the round before slab k + 1 starts.  Every cell of plane z then
+// takes step s after planes z - 1 and z + 1 have taken step s - 1 and before
+// either takes step s + 1.  That is all the in-place update needs (the slots
+// that a cell's step s touches are touched only by the cell's and its
+// neighbours' steps s - 1 and s + 1), so results do not depend on the plan.
+// In a box periodic in z the first slab moves up at its bottom,
+// [s, begin(1) - s), and the last one ends with the planes that this leaves:
+// past the top and round to plane s - 1.
+struct SlabPlan {
+  int slabs = 1;
+  int depth = 1;  // steps of a round
+};
+
+// The slabs of d's steps on a device with l2_bytes of L2.
+SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes);
+
+// launch(s, z0, planes) for every step s of 0 .. count - 1 and slab.
+template <typename Fn>
+cudaError_t run_slabs(int nz, bool periodic, const SlabPlan& plan, int64_t count, Fn&& launch) {
+  // begin(k) leaves every slab the same number of planes per round: (planes
+  // to share out) / slabs, plus the depth-wide ramp at the bottom
+  const int64_t share = periodic ? nz : nz - plan.depth;
+  auto begin = [&](int k) { return k == 0 ? 0 : plan.depth + (int)(k * share / plan.slabs); };
+  for (int64_t s0 = 0; s0 < count; s0 += plan.depth) {
+    const int steps = (int)(count - s0 < plan.depth ? count - s0 : plan.depth);
+    // two or three steps do not save what the extra launches cost
+    const int slabs = steps >= 4 ? plan.slabs : 1;
+    for (int k = 0; k < slabs; ++k)
+      for (int s = 0; s < steps; ++s) {
+        int lo = k == 0 ? 0 : begin(k) - s;
+        int hi = k == slabs - 1 ? nz : begin(k + 1) - s;
+        if (periodic && slabs > 1) {
+          if (k == 0) lo = s;
+          if (k == slabs - 1) hi = nz + s;
+        }
+        if (cudaError_t e = launch(s0 + s, lo, hi - lo)) return e;
+      }
+  }
+  return cudaSuccess;
+}
+
 // Queue the fused steps n .. n + count - 1 (parity of each its number's).
 cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                         cudaStream_t st);
+                         const SlabPlan& plan, cudaStream_t st);
 
 // f = f_eq(p - p_ref, u) at every node, stored for step 0 (even layout).
 cudaError_t launch_init(const DomainDesc& d, const double* u, const double* p,

@@ -25,6 +25,7 @@ template <typename R>
 struct Domain {
   void* f;           // population buffer, Q*N values of the storage type
   int nx, ny, nz;
+  int z0;            // first plane of this launch (launches over a slab of planes)
   int64_t N;         // nx*ny*nz
   int per[3];        // axis is periodic
   int moving;        // bit f set: face f is a moving wall
@@ -127,6 +128,14 @@ __host__ __device__ inline void fill_offsets(Domain<R>& d) {
         }(),
         ...);
   }(std::make_integer_sequence<int, Q>{});
+}
+
+// Plane of the calling CTA in a launch of gridDim.z planes from d.z0 on; past
+// the last plane it goes on at plane 0 (slabs of a box periodic in z).
+template <typename R>
+__device__ __forceinline__ int slab_plane(const Domain<R>& d) {
+  const int z = d.z0 + (int)blockIdx.z;
+  return z < d.nz ? z : z - d.nz;
 }
 
 // Edge-profile factor of moving face `face` for a cell whose position bits

@@ -1,6 +1,7 @@
 // Single-domain step: descriptor conversion, force time level, default launch
 // shape, and dispatch to the per-Q kernel files (lbm_step_q14.cu, _q18.cu,
 // _q26.cu).
+#include <algorithm>
 #include <cmath>
 
 #include "lbm_internal.h"
@@ -90,6 +91,36 @@ const char* set_faces(DomainDesc& d, const lbm_geom* g) {
   return nullptr;
 }
 
+// When and how a box is swept in slabs.  Measured on D3Q18 FP32 boxes of
+// 128 x 128 x nz (135 MB of L2): a sweep of the whole box runs at 60-62 GLUPS
+// up to 76 MB of populations, 57 at 85, 52 at 94, 45 at 113 and 44 from 150 MB
+// on, where every step goes to memory; slabs run at 56-58 throughout (nz = 128:
+// 47.7 us a step in whole sweeps, 37.1 in slabs).  They pay from about 0.65
+// of L2 on.  A slab may touch 0.62 of L2: 128^3 takes 37.1 us with 66-78 MB a
+// slab, 39.4 with 55 or 90 MB; 256^3 takes 326 with 85, 331 with 75, 360 in
+// whole sweeps.  A round is 3/8 of the planes a slab touches, at most 16: the
+// round's steps share one trip to memory, but each costs the slab a plane and
+// every launch about 2 us of ramp and tail (128^3: 4 steps 40.4 us, 8 38.1,
+// 16 37.1, 32 37.4).  Fewer than 10 planes (boxes of 350^2 and more) leave
+// nothing to gain (320^3: 693 us against 700).  The other storage types are
+// not bound by memory in a whole sweep: FP64 by its arithmetic, FP16 and BF16
+// by their issue rate (256^3 D3Q18 FP16: 232 us in whole sweeps, 240 in slabs).
+SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
+  if (d.storage != LBM_STORAGE_F32) return {};
+  const int64_t plane = (int64_t)d.nx * d.ny * (d.Q * 4 + (d.solid ? 4 : 0));
+  if (plane * d.nz * 100 < l2_bytes * 65) return {};
+  const int touched = (int)std::min<int64_t>(l2_bytes * 62 / 100 / plane, d.nz);
+  if (touched < 10) return {};
+  SlabPlan p;
+  p.depth = std::min(16, touched * 3 / 8);
+  const int own = touched - p.depth, share = d.per[2] ? d.nz : d.nz - p.depth;
+  p.slabs = (share + own - 1) / own;
+  // every slab keeps a plane, also while the first one of a periodic box
+  // shrinks from both sides
+  if (p.slabs < 2 || share / p.slabs <= p.depth) return {};
+  return p;
+}
+
 BlockShape default_block(int nx, int ny) {
   int bx = 32;
   while (bx < nx && bx < 128) bx *= 2;
@@ -99,18 +130,18 @@ BlockShape default_block(int nx, int ny) {
 }
 
 cudaError_t launch_step_q14(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st);
 cudaError_t launch_step_q18(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st);
 cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st);
 
 cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                         cudaStream_t st) {
+                         const SlabPlan& plan, cudaStream_t st) {
   if (d.N == 0) return cudaSuccess;
-  if (d.Q == 14) return launch_step_q14(d, n, count, b, st);
-  if (d.Q == 18) return launch_step_q18(d, n, count, b, st);
-  if (d.Q == 26) return launch_step_q26(d, n, count, b, st);
+  if (d.Q == 14) return launch_step_q14(d, n, count, b, plan, st);
+  if (d.Q == 18) return launch_step_q18(d, n, count, b, plan, st);
+  if (d.Q == 26) return launch_step_q26(d, n, count, b, plan, st);
   return cudaErrorInvalidValue;
 }
 

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
   pdl_acquire();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
+  const int z = slab_plane(d);
   if (x >= d.nx || y >= d.ny) return;
   // a 32-wide x-range containing x; it is the calling warp's range when
   // blockDim.x is a multiple of 32 (then the path choice is warp-uniform)
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256, 3) k_step_pair(Domain<float> d) {
   pdl_acquire();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
+  const int z = slab_plane(d);
   if (x0 >= d.nx || y >= d.ny) return;
   update_pair_even<Q, S, FORCE, SR>(d, static_cast<S*>(d.f), x0 + d.nx * (y + d.ny * z));
 }
@@ -104,36 +104,36 @@ void launch_parity(const Domain<R>& d, bool odd, bool force, bool wide, dim3 gri
   }
 }
 
-// Steps n .. n + count - 1.  The descriptor is built once; a launch changes
-// only its force and rounding key, so it costs the host 1.8 us where
-// rebuilding the descriptor made it 5.5 us (16^3 D3Q18 FP32: 6.0 us a step
-// before, 2.0 us now).
+// Steps n .. n + count - 1, slab by slab (run_slabs).  The descriptor is
+// built once; a launch changes only its planes, force and rounding key, so it
+// costs the host 1.8 us where rebuilding the descriptor made it 5.5 us (16^3
+// D3Q18 FP32: 6.0 us a step before, 2.0 us now).
 template <int Q, typename S, typename R>
 cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockShape b,
-                         cudaStream_t st) {
+                         const SlabPlan& plan, cudaStream_t st) {
   const double zero[3] = {0.0, 0.0, 0.0};
   // the force-carrying update whenever the amplitude is nonzero (also at the
   // steps where a periodic force passes through zero), as the batch does
   const bool force = dd.force[0] != 0.0 || dd.force[1] != 0.0 || dd.force[2] != 0.0;
   Domain<R> d = to_domain<R>(dd, zero);
   const dim3 block(b.bx, b.by, 1);
-  const dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, dd.nz);
   const bool wide = (int64_t)dd.Q * dd.N >= (int64_t(1) << 31);
   bool sr = false;
   if constexpr (Stochastic<S>::enabled) sr = dd.rounding == LBM_ROUND_STOCHASTIC;
-  for (int64_t k = n; k < n + count; ++k) {
+  return run_slabs(dd.nz, dd.per[2] != 0, plan, count, [&](int64_t s, int z0, int planes) {
     double F[3];
-    force_at(dd, k, F);
+    force_at(dd, n + s, F);
     for (int c = 0; c < 3; ++c) d.F[c] = R(F[c]);
-    d.key = step_key(k);
-    const bool odd = (k & 1) != 0;
+    d.key = step_key(n + s);
+    d.z0 = z0;
+    const dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, planes);
+    const bool odd = ((n + s) & 1) != 0;
     if constexpr (Stochastic<S>::enabled) {
       if (sr) launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
     }
     if (!sr) launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
-    if (cudaError_t e = cudaGetLastError()) return e;
-  }
-  return cudaSuccess;
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace lbm

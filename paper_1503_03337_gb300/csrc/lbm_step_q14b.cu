@@ -4,8 +4,8 @@
 namespace lbm {
 
 cudaError_t launch_step_q14_bf16(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                                 cudaStream_t st) {
-  return launch_typed<14, __nv_bfloat16, float>(d, n, count, b, st);
+                                 const SlabPlan& plan, cudaStream_t st) {
+  return launch_typed<14, __nv_bfloat16, float>(d, n, count, b, plan, st);
 }
 
 }  // namespace lbm

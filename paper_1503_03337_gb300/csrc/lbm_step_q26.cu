@@ -6,15 +6,15 @@
 namespace lbm {
 
 cudaError_t launch_step_q26_half(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                                 cudaStream_t st);
+                                 const SlabPlan& plan, cudaStream_t st);
 
 cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            cudaStream_t st) {
+                            const SlabPlan& plan, cudaStream_t st) {
   switch (d.storage) {
-    case LBM_STORAGE_F64: return launch_typed<26, double, double>(d, n, count, b, st);
-    case LBM_STORAGE_F32: return launch_typed<26, float, float>(d, n, count, b, st);
+    case LBM_STORAGE_F64: return launch_typed<26, double, double>(d, n, count, b, plan, st);
+    case LBM_STORAGE_F32: return launch_typed<26, float, float>(d, n, count, b, plan, st);
     case LBM_STORAGE_F16:
-    case LBM_STORAGE_BF16: return launch_step_q26_half(d, n, count, b, st);
+    case LBM_STORAGE_BF16: return launch_step_q26_half(d, n, count, b, plan, st);
   }
   return cudaErrorInvalidValue;
 }
