@@ -46,7 +46,7 @@ struct BlockShape {
   int pdl = 1;  // programmatic dependent launch of consecutive steps
 };
 
-BlockShape default_block(int nx, int ny);
+BlockShape default_block(int nx, int ny, int storage);
 
 // The face fields of d (per, moving, sym, neq_*, uw) from a geometry.
 // Returns nullptr, or the reason the geometry is invalid (then d is

@@ -121,7 +121,8 @@ SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
   return p;
 }
 
-BlockShape default_block(int nx, int ny) {
+BlockShape default_block(int nx, int ny, int storage) {
+  if (storage == LBM_STORAGE_F64) return {32, 1, 1};  // one warp each (k_step_f64)
   int bx = 32;
   while (bx < nx && bx < 128) bx *= 2;
   int by = 256 / bx;

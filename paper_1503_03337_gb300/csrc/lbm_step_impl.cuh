@@ -45,6 +45,40 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
                                                     x_hi);
 }
 
+// FP64 storage: cells in linear order, one after another whatever row they
+// are in.  This device updates two FP64 lanes per clock and SM, so a warp
+// instruction takes 16 clocks however many of its lanes are active, and the
+// step is bound by that pipe; rows rounded up to whole warps waste it (16-wide
+// rows half of it, 65-wide ones a third), as does any branch that splits a
+// warp, so every cell takes the general addressing.  Launched with one warp
+// per block (default_block): the warps then spread evenly over the SMs.
+// 16x16x32 D3Q18: 30.8 us a step with 32 x 8 blocks of rows, 8.2 so; 65x33x33
+// D3Q14: 30 and 14.
+template <int Q, bool ODD, bool FORCE, bool WIDE>
+__global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(Domain<double> d) {
+  pdl_release();
+  pdl_acquire();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // N < 2^31
+  if (t >= (unsigned)d.N) return;
+  const int i = (int)t;
+  double* const f = static_cast<double*>(d.f);
+  if constexpr (!ODD) {
+    if (d.solid && (d.solid[i] & kSolidCell)) return;
+    update_with_links<Q, double, double, false, FORCE, false, false, true, false, WIDE>(
+        d, f, i, Links{}, d.F, &d.key);
+  } else {
+    const int x = i % d.nx, r = i / d.nx;
+    const Links L = make_links(d, x, r % d.ny, r / d.ny);
+    if (L.solid & kSolidCell) return;
+    if (d.sym)
+      update_with_links<Q, double, double, true, FORCE, false, false, true, true, WIDE>(
+          d, f, i, L, d.F, &d.key);
+    else
+      update_with_links<Q, double, double, true, FORCE, false, false, false, true, WIDE>(
+          d, f, i, L, d.F, &d.key);
+  }
+}
+
 // Even steps with two x-adjacent cells per thread (see update_pair_even; nx
 // even); blockDim.x threads cover 2*blockDim.x cells of a row.  The 36
 // packed values of a pair need more registers than one cell's 18: at three
@@ -67,6 +101,22 @@ template <typename R>
 void launch_one(void (*kernel)(Domain<R>), const Domain<R>& d, dim3 grid, dim3 block, bool pdl,
                 cudaStream_t st) {
   launch_pdl(kernel, grid, block, pdl, st, d);
+}
+
+template <int Q>
+void launch_f64(const Domain<double>& d, bool odd, bool force, bool wide, const BlockShape& b,
+                cudaStream_t st) {
+  auto kernel = wide ? (odd ? (force ? k_step_f64<Q, true, true, true>
+                                     : k_step_f64<Q, true, false, true>)
+                            : (force ? k_step_f64<Q, false, true, true>
+                                     : k_step_f64<Q, false, false, true>))
+                     : (odd ? (force ? k_step_f64<Q, true, true, false>
+                                     : k_step_f64<Q, true, false, false>)
+                            : (force ? k_step_f64<Q, false, true, false>
+                                     : k_step_f64<Q, false, false, false>));
+  const unsigned threads = b.bx * b.by;
+  launch_one(kernel, d, dim3((unsigned)((d.N + threads - 1) / threads)), dim3(threads),
+             b.pdl != 0, st);
 }
 
 template <int Q, typename S, typename R, bool SR>
@@ -128,10 +178,14 @@ cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockSh
     d.z0 = z0;
     const dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, planes);
     const bool odd = ((n + s) & 1) != 0;
-    if constexpr (Stochastic<S>::enabled) {
-      if (sr) launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
+    if constexpr (sizeof(S) == 8) {
+      launch_f64<Q>(d, odd, force, wide, b, st);
+    } else {
+      if constexpr (Stochastic<S>::enabled) {
+        if (sr) launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
+      }
+      if (!sr) launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
     }
-    if (!sr) launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
     return cudaGetLastError();
   });
 }
