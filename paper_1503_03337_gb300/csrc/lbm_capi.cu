@@ -404,7 +404,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     h->n += m;
     nsteps -= m;
     if (neq) {  // the extrapolation boundaries of the new time level
-      e = launch_neq(h->d, h->n, h->stream);
+      e = launch_neq(h->d, h->n, h->block.pdl != 0, h->stream);
       if (e != cudaSuccess) return cuda_fail(e, "boundary kernel");
     }
     if (K > 0 && h->n % K == 0)

@@ -60,7 +60,7 @@ cudaError_t launch_solid_links(const DomainDesc& d, const uint8_t* bytes, uint32
 
 // Non-equilibrium extrapolation of the boundary nodes of d's LBM_NEQ_*
 // faces, on the populations of step n (after the step n-1 -> n).
-cudaError_t launch_neq(const DomainDesc& d, int64_t n, cudaStream_t st);
+cudaError_t launch_neq(const DomainDesc& d, int64_t n, bool pdl, cudaStream_t st);
 
 // Message returned by lbm_last_error() on the calling thread.
 void set_last_error(const std::string& msg);

@@ -110,6 +110,43 @@ __host__ __device__ constexpr int pair_rep(int i) {
   return -1;
 }
 
+// fn.operator()<A, B>() for every pair of opposite directions A < B.
+template <int Q, typename Fn>
+__host__ __device__ __forceinline__ void for_pairs(Fn&& fn) {
+  [&]<int... I>(std::integer_sequence<int, I...>) {
+    (fn.template operator()<pair_rep<Q>(I), opposite<Q>(pair_rep<Q>(I))>(), ...);
+  }(std::make_integer_sequence<int, Q / 2>{});
+}
+
+// acc + C v for C = -1, 0, 1 (multiplying by a constant zero would stay)
+template <int C, typename R>
+__host__ __device__ __forceinline__ R add_signed(R acc, R v) {
+  if constexpr (C > 0) return acc + v;
+  else if constexpr (C < 0) return acc - v;
+  else return acc;
+}
+// c . v of direction A
+template <int Q, int A, typename R>
+__host__ __device__ __forceinline__ R dot_c(const R* v) {
+  constexpr int cx = Lattice<Q>::c(A, 0), cy = Lattice<Q>::c(A, 1), cz = Lattice<Q>::c(A, 2);
+  if constexpr (cx != 0) return add_signed<cz>(add_signed<cy>(cx > 0 ? v[0] : -v[0], v[1]), v[2]);
+  else if constexpr (cy != 0) return add_signed<cz>(cy > 0 ? v[1] : -v[1], v[2]);
+  else return cz > 0 ? v[2] : -v[2];
+}
+
+// P = sum f and j = sum c f of one cell, from the pair sums and differences.
+template <int Q, typename R>
+__host__ __device__ __forceinline__ void pair_moments(const R* f, R& P, R* j) {
+  P = j[0] = j[1] = j[2] = R(0);
+  for_pairs<Q>([&]<int A, int B>() {
+    const R diff = f[A] - f[B];
+    P += f[A] + f[B];
+    j[0] = add_signed<Lattice<Q>::c(A, 0)>(j[0], diff);
+    j[1] = add_signed<Lattice<Q>::c(A, 1)>(j[1], diff);
+    j[2] = add_signed<Lattice<Q>::c(A, 2)>(j[2], diff);
+  });
+}
+
 // ---------------------------------------------------------------------------
 // Moment basis
 // ---------------------------------------------------------------------------

@@ -46,34 +46,35 @@ __host__ __device__ inline void neq_node(const Domain<R>& d, const NeqArgs& a, i
   }
   R fv[Q];
   get_canonical<Q, S, R, ODD>(d, static_cast<const S*>(d.f), xf[0], xf[1], xf[2], fv);
-  R P = R(0), uf[3] = {R(0), R(0), R(0)};
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    P += fv[q];
-    uf[0] += R(Lattice<Q>::c(q, 0)) * fv[q];
-    uf[1] += R(Lattice<Q>::c(q, 1)) * fv[q];
-    uf[2] += R(Lattice<Q>::c(q, 2)) * fv[q];
-  }
+  R P, uf[3];
+  pair_moments<Q>(fv, P, uf);
   for (int c = 0; c < 3; ++c) uf[c] += R(0.5) * d.F[c];
   // Eq. hgl: p = c_s^2 / (1 - w0) (P - w0 |u|^2 / (2 c_s^2)), c_s^2 = 1/3
   constexpr double w0 = Lattice<Q>::w0;
   const R uf2 = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
   const R pf = R(1.0 / (3.0 * (1.0 - w0))) * (P - R(1.5 * w0) * uf2);
-  R ub[3], pb;
-  for (int c = 0; c < 3; ++c) ub[c] = vel_face >= 0 ? d.uw[vel_face][c] : uf[c];
-  pb = pre_face >= 0 ? R(a.pb[pre_face]) : pf;
-  const R ub2 = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const R cx = R(Lattice<Q>::c(q, 0)), cy = R(Lattice<Q>::c(q, 1)), cz = R(Lattice<Q>::c(q, 2));
-    const R w = R(Lattice<Q>::w(q));
-    const R cub = cx * ub[0] + cy * ub[1] + cz * ub[2];
-    const R cuf = cx * uf[0] + cy * uf[1] + cz * uf[2];
-    // Eq. edf: f_eq = w (3 p + 3 c.u + 9/2 (c.u)^2 - 3/2 |u|^2)
-    const R eb = w * (R(3) * pb + R(3) * cub + R(4.5) * cub * cub - R(1.5) * ub2);
-    const R ef = w * (R(3) * pf + R(3) * cuf + R(4.5) * cuf * cuf - R(1.5) * uf2);
-    fv[q] = eb + (fv[q] - ef);
+  // With Eq. edf, f_eq = w (3 p + 3 c.u + 9/2 (c.u)^2 - 3/2 |u|^2), and
+  // du = u_b - u_f, su = u_b + u_f:
+  //   f_eq(p_b, u_b) - f_eq(p_f, u_f) = w (3 (p_b - p_f) - 3/2 du.su
+  //                                        + 3 c.du + 9/2 (c.du) (c.su)),
+  // whose odd part 3 w c.du only changes sign between opposite populations.
+  // Forming the difference this way takes a third of the operations of the
+  // two equilibria, which bound the pass with FP64 storage.
+  R du[3], su[3];
+  for (int c = 0; c < 3; ++c) {
+    const R ub = vel_face >= 0 ? d.uw[vel_face][c] : uf[c];
+    du[c] = ub - uf[c];
+    su[c] = ub + uf[c];
   }
+  const R dp = pre_face >= 0 ? R(a.pb[pre_face]) - pf : R(0);
+  const R base = R(3) * dp - R(1.5) * (du[0] * su[0] + du[1] * su[1] + du[2] * su[2]);
+  for_pairs<Q>([&]<int A, int B>() {
+    const R cd = dot_c<Q, A>(du), cs = dot_c<Q, A>(su);
+    const R even = R(Lattice<Q>::w(A)) * (base + R(4.5) * cd * cs);
+    const R odd = R(3.0 * Lattice<Q>::w(A)) * cd;
+    fv[A] += even + odd;
+    fv[B] += even - odd;
+  });
   put_canonical<Q, S, R, ODD>(d, static_cast<S*>(d.f), xyz[0], xyz[1], xyz[2], fv);
 }
 

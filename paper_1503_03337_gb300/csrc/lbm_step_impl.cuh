@@ -52,8 +52,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
 // rows half of it, 65-wide ones a third), as does any branch that splits a
 // warp, so every cell takes the general addressing.  Launched with one warp
 // per block (default_block): the warps then spread evenly over the SMs.
-// 16x16x32 D3Q18: 30.8 us a step with 32 x 8 blocks of rows, 8.2 so; 65x33x33
-// D3Q14: 30 and 14.
+// 16x16x32 D3Q18: 30.8 us a step with 32 x 8 blocks of rows, 8.2 so.
 template <int Q, bool ODD, bool FORCE, bool WIDE>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(Domain<double> d) {
   pdl_release();
