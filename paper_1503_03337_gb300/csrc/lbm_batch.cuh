@@ -77,8 +77,8 @@ __device__ __forceinline__ void batch_tile(const Domain<float>& d, int tx, int t
   const int y = ty * blockDim.y + threadIdx.y;
   if (x >= d.nx || y >= d.ny) return;
   const int x_lo = tx * blockDim.x + (threadIdx.x & ~31);
-  update_cell<Q, S, float, ODD, FORCE, SR, CG>(d, static_cast<S*>(d.f), x, y, z, x_lo,
-                                               x_lo + 31);
+  update_cell<Q, S, float, ODD, FORCE, SR, CG, false, false>(d, static_cast<S*>(d.f), x, y, z,
+                                                             x_lo, x_lo + 31);
 }
 
 // Walks the tiles of one domain in order (x fastest) without divisions.
@@ -211,10 +211,11 @@ __global__ void __launch_bounds__(256, DYN ? 3 : 4)
   if (x >= d.nx || y >= d.ny) return;
   const int x_lo = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   if constexpr (DYN)
-    update_cell_at<Q, S, float, ODD, FORCE, SR>(d, static_cast<S*>(d.f), dyn->F, &dyn->key, x,
-                                                y, z, x_lo, x_lo + 31);
+    update_cell_at<Q, S, float, ODD, FORCE, SR, false, false, false>(
+        d, static_cast<S*>(d.f), dyn->F, &dyn->key, x, y, z, x_lo, x_lo + 31);
   else
-    update_cell<Q, S, float, ODD, FORCE, SR>(d, static_cast<S*>(d.f), x, y, z, x_lo, x_lo + 31);
+    update_cell<Q, S, float, ODD, FORCE, SR, false, false, false>(d, static_cast<S*>(d.f), x, y,
+                                                                  z, x_lo, x_lo + 31);
 }
 
 // Launch of one group's grouped kernel for one step (per-Q files).

@@ -393,7 +393,9 @@ __host__ __device__ __forceinline__ void gather(const Domain<R>& d, const S* __r
     }(std::make_integer_sequence<int, Q>{});
   } else if (L.interior) {
     [&]<int... A>(std::integer_sequence<int, A...>) {
-      ((fv[A] = load_pop<S, R, CG>(fc + pull_offset<WIDE>(d, A))), ...);
+      ((fv[A] = load_pop<S, R, CG>(fc + (SOLID && ((L.solid >> A) & 1u) ? A * N
+                                                                        : pull_offset<WIDE>(d, A)))),
+       ...);
     }(std::make_integer_sequence<int, Q>{});
   } else {
     // f_a(x) = A[abar][x - c_a], or A[a][x] if x - c_a is a wall ghost;
@@ -474,7 +476,10 @@ __host__ __device__ __forceinline__ void scatter(const Domain<R>& d, S* __restri
   if constexpr (!ODD) {
     store_cell<Q, S, R, SR>(fv, h, [&]<int A>() { return fc + (size_t)opposite<Q>(A) * d.N; });
   } else if (L.interior) {
-    store_cell<Q, S, R, SR>(fv, h, [&]<int A>() { return fc + push_offset<WIDE>(d, A); });
+    store_cell<Q, S, R, SR>(fv, h, [&]<int A>() {
+      constexpr int B = opposite<Q>(A);
+      return fc + (SOLID && ((L.solid >> B) & 1u) ? B * N : push_offset<WIDE>(d, A));
+    });
   } else {
     if (d.moving && touches_moving(d, L)) {
       [&]<int... A>(std::integer_sequence<int, A...>) {
@@ -534,24 +539,41 @@ __host__ __device__ __forceinline__ bool warp_any(bool v) {
 // across the grid), so domains without one pay nothing for them.
 // update_cell_at reads the step's body force F[0..2] and rounding key *key
 // where they are used (F and key may live outside the descriptor);
-// update_cell takes them from the descriptor.
+// update_cell takes them from the descriptor.  SOLIDS = false: the domain has
+// no solid mask (batched domains).
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,
-          bool CG = false, bool WIDE = false>
+          bool CG = false, bool WIDE = false, bool SOLIDS = true>
 __host__ __device__ __forceinline__ void update_cell_at(const Domain<R>& d, S* __restrict__ f,
                                                         const R* F, const uint32_t* key, int x,
                                                         int y, int z, int x_lo, int x_hi) {
   const int i = x + d.nx * (y + d.ny * z);
   if constexpr (!ODD) {
-    if (d.solid && (d.solid[i] & kSolidCell)) return;  // solid cells hold no flow
+    if (SOLIDS && d.solid && (d.solid[i] & kSolidCell)) return;  // solid cells hold no flow
     Links L{};
     update_with_links<Q, S, R, false, FORCE, SR, CG, true, false, WIDE>(d, f, i, L, F, key);
   } else {
-    if (d.solid) {
+    if (SOLIDS && d.solid) {
       // a warp with any solid-touching link takes the full addressing with
       // the cells' solid bits (the vote comes before any lane leaves)
       const uint32_t sm = d.solid[i];
       if (warp_any(sm != 0u)) {
         if (sm & kSolidCell) return;
+        // In the bulk only the solid bits redirect a link: one select between
+        // two tabled offsets, or the x-only addressing, instead of the full
+        // one (porous 192^3, 30 % solid, D3Q18 FP32: 153 us a step before, 141
+        // now).
+        if (!d.sym && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
+          if (x_lo > 0 && x_hi < d.nx - 1) {
+            Links L = make_links_interior(d);
+            L.solid = sm;
+            update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
+          } else {
+            Links L = make_links_x(d, x);
+            L.solid = sm;
+            update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
+          }
+          return;
+        }
         if (d.sym)
           update_with_links<Q, S, R, true, FORCE, SR, CG, true, true, WIDE>(
               d, f, i, make_links(d, x, y, z), F, key);
@@ -582,11 +604,11 @@ __host__ __device__ __forceinline__ void update_cell_at(const Domain<R>& d, S* _
 }
 
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,
-          bool CG = false, bool WIDE = false>
+          bool CG = false, bool WIDE = false, bool SOLIDS = true>
 __host__ __device__ __forceinline__ void update_cell(const Domain<R>& d, S* __restrict__ f,
                                                      int x, int y, int z, int x_lo = -1,
                                                      int x_hi = -1) {
-  update_cell_at<Q, S, R, ODD, FORCE, SR, CG, WIDE>(d, f, d.F, &d.key, x, y, z, x_lo, x_hi);
+  update_cell_at<Q, S, R, ODD, FORCE, SR, CG, WIDE, SOLIDS>(d, f, d.F, &d.key, x, y, z, x_lo, x_hi);
 }
 
 // Two storage values of x-adjacent cells as one word (8 bytes for FP32,
