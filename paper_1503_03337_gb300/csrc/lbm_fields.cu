@@ -152,33 +152,38 @@ struct ReduceArgs {
   double edge_scale[6][2];  // their edge profiles (Domain::edge_scale)
 };
 
-__device__ __forceinline__ void block_reduce(double (&v)[kNumStats], double* shm) {
-  // warp level
+// Blocks of a reduction: four resident ones per SM, each looping over cells,
+// so that the FP64 end of a block is paid four times an SM.
+constexpr int kReduceGrid = 608;
+static_assert(kReduceGrid <= kReduceBlocks, "partials buffer");
+
+// The block's statistics from every thread's v, to partials[k * gridDim.x +
+// blockIdx.x].  FP64 adds run at two lanes per clock and SM, so their number
+// is what this costs: the threads' values are laid out in shared memory and
+// one warp sums statistic k, 32 lanes of a few values each and five shuffles
+// (180 warp adds a block of 256 threads; reducing all fifteen by shuffles in
+// every warp took 700 and 5 us a block, on eight blocks an SM).
+__device__ __forceinline__ void block_partials(const double (&v)[kNumStats], double* partials) {
+  __shared__ double shm[kNumStats][kReduceThreads];
 #pragma unroll
-  for (int k = 0; k < kNumStats; ++k) {
+  for (int k = 0; k < kNumStats; ++k) shm[k][threadIdx.x] = v[k];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < kNumStats; k += kReduceThreads / 32) {
+    double t = shm[k][lane];
+    for (int j = lane + 32; j < kReduceThreads; j += 32)
+      t = k == kNumSums ? fmax(t, shm[k][j]) : t + shm[k][j];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double t = __shfl_down_sync(0xffffffffu, v[k], o);
-      v[k] = (k == kNumSums) ? fmax(v[k], t) : v[k] + t;
+      const double w = __shfl_down_sync(0xffffffffu, t, o);
+      t = k == kNumSums ? fmax(t, w) : t + w;
     }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  if (lane == 0)
-    for (int k = 0; k < kNumStats; ++k) shm[warp * kNumStats + k] = v[k];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < nwarps; ++w)
-      for (int k = 0; k < kNumStats; ++k) {
-        const double t = shm[w * kNumStats + k];
-        v[k] = (k == kNumSums) ? fmax(v[k], t) : v[k] + t;
-      }
+    if (lane == 0) partials[k * gridDim.x + blockIdx.x] = t;
   }
 }
 
 template <int Q, typename S, bool ODD>
 __global__ void __launch_bounds__(kReduceThreads) k_reduce(Domain<double> d, ReduceArgs a) {
-  __shared__ double shm[(kReduceThreads / 32) * kNumStats];
   double v[kNumStats];
   for (int k = 0; k < kNumStats; ++k) v[k] = 0.0;
   const int64_t N = d.N;
@@ -211,9 +216,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(Domain<double> d, Red
     }
     v[9] += P + 3.0 * (1.0 - Lattice<Q>::w0) * a.p_ref;
   }
-  block_reduce(v, shm);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kNumStats; ++k) a.partials[blockIdx.x * kNumStats + k] = v[k];
+  block_partials(v, a.partials);
 }
 
 // A value kept as the unevaluated pair hi + lo of FP32 numbers.  Each
@@ -326,7 +329,6 @@ template <int Q, typename S, bool ODD, bool WIDE>
 __global__ void __launch_bounds__(kReduceThreads) k_reduce_pair(Domain<float> d, ReduceArgs a,
                                                                  PairSum Fh0, PairSum Fh1,
                                                                  PairSum Fh2, PairSum Pref) {
-  __shared__ double shm[(kReduceThreads / 32) * kNumStats];
   PairSum sdu[3], su_abs[3], sup_abs[3], su[3], sPt, umax;
   int nonfinite = 0;
   const PairSum Fh[3] = {Fh0, Fh1, Fh2};
@@ -390,25 +392,25 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_pair(Domain<float> d,
   v[9] = value_of(sPt);
   v[kNumSums - 1] = (double)nonfinite;
   v[kNumSums] = value_of(umax);
-  block_reduce(v, shm);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kNumStats; ++k) a.partials[blockIdx.x * kNumStats + k] = v[k];
+  block_partials(v, a.partials);
 }
 
-// Sums the per-block partials in a fixed order (deterministic result).
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_final(const double* partials,
+// Sums the per-block partials in a fixed order (deterministic result): one
+// warp per statistic.
+__global__ void __launch_bounds__(32 * kNumStats) k_reduce_final(const double* partials,
                                                                  int nblocks, double* out) {
-  __shared__ double shm[(kReduceThreads / 32) * kNumStats];
-  double v[kNumStats];
-  for (int k = 0; k < kNumStats; ++k) v[k] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-    for (int k = 0; k < kNumStats; ++k) {
-      const double t = partials[b * kNumStats + k];
-      v[k] = (k == kNumSums) ? fmax(v[k], t) : v[k] + t;
-    }
-  block_reduce(v, shm);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kNumStats; ++k) out[k] = v[k];
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double t = 0.0;
+  for (int b = lane; b < nblocks; b += 32) {
+    const double w = partials[k * nblocks + b];
+    t = k == kNumSums ? fmax(t, w) : t + w;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_down_sync(0xffffffffu, t, o);
+    t = k == kNumSums ? fmax(t, w) : t + w;
+  }
+  if (lane == 0) out[k] = t;
 }
 
 int grid_for(int64_t N) {
@@ -515,7 +517,7 @@ cudaError_t launch_reduce(const DomainDesc& dd, int64_t n, double* u_prev, int h
     for (int k = 0; k < 2; ++k) a.edge_scale[face][k] = dd.edge_scale[face][k];
   }
   int64_t g = (dd.N + kReduceThreads - 1) / kReduceThreads;
-  if (g > kReduceBlocks) g = kReduceBlocks;
+  if (g > kReduceGrid) g = kReduceGrid;
   if (g < 1) g = 1;
   const bool odd = n & 1;
   const Domain<float> df = to_domain<float>(dd, F);
@@ -535,7 +537,7 @@ cudaError_t launch_reduce(const DomainDesc& dd, int64_t n, double* u_prev, int h
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
-  k_reduce_final<<<1, kReduceThreads, 0, st>>>(partials, (int)g, out);
+  k_reduce_final<<<1, 32 * kNumStats, 0, st>>>(partials, (int)g, out);
   return cudaGetLastError();
 }
 
