@@ -190,7 +190,7 @@ int lbm_create(const lbm_desc* desc, void* cuda_stream, lbm_handle** out) {
   h->d.nz = desc->nz;
   h->d.storage = desc->storage;
   h->d.N = N;
-  h->block = default_block(desc->nx, desc->ny, desc->storage);
+  h->block = default_block(desc->nx, desc->ny, N, desc->storage);
 
   const size_t fbytes = (size_t)N * desc->Q * b;
   e = cudaMalloc(&h->d.f, fbytes);

@@ -46,7 +46,27 @@ struct BlockShape {
   int pdl = 1;  // programmatic dependent launch of consecutive steps
 };
 
-BlockShape default_block(int nx, int ny, int storage);
+// i / n for 0 <= i < 2^31 and n >= 1 as a multiplication: with n <= 2^s < 2 n
+// and m = floor(2^(31+s) / n) + 1 < 2^32, i m >> (31 + s) is exact because
+// i (m n - 2^(31+s)) <= i 2^s < 2^(31+s).
+struct FastDiv {
+  unsigned m;
+  int shift;
+  explicit FastDiv(int n) {
+    int s = 0;
+    while ((int64_t(1) << s) < n) ++s;
+    m = (unsigned)((uint64_t(1) << (31 + s)) / (unsigned)n + 1);
+    shift = 31 + s;
+  }
+  __host__ __device__ int operator()(int i) const {
+    return (int)(((uint64_t)(unsigned)i * m) >> shift);
+  }
+};
+
+// The default launch of a box; 4- and 2-byte storage runs its cells in linear
+// order (k_step_line) or by rows (k_step).
+BlockShape default_block(int nx, int ny, int64_t N, int storage);
+bool steps_in_line(int nx, int ny, int64_t N);
 
 // The face fields of d (per, moving, sym, neq_*, uw) from a geometry.
 // Returns nullptr, or the reason the geometry is invalid (then d is

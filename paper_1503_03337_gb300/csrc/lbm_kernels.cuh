@@ -541,66 +541,84 @@ __host__ __device__ __forceinline__ bool warp_any(bool v) {
 // where they are used (F and key may live outside the descriptor);
 // update_cell takes them from the descriptor.  SOLIDS = false: the domain has
 // no solid mask (batched domains).
+
+// Even step of cell i: its own slots only.
+template <int Q, typename S, typename R, bool FORCE, bool SR, bool CG, bool WIDE, bool SOLIDS>
+__host__ __device__ __forceinline__ void update_even(const Domain<R>& d, S* __restrict__ f,
+                                                     const R* F, const uint32_t* key, int i) {
+  if (SOLIDS && d.solid && (d.solid[i] & kSolidCell)) return;  // solid cells hold no flow
+  Links L{};
+  update_with_links<Q, S, R, false, FORCE, SR, CG, true, false, WIDE>(d, f, i, L, F, key);
+}
+
+// Odd step of cell i = (x, y, z); bulk_yz: no cell of the warp lies on a y or
+// z face, bulk_x: none at a row end (both uniform across the warp).
+template <int Q, typename S, typename R, bool FORCE, bool SR, bool CG, bool WIDE, bool SOLIDS>
+__host__ __device__ __forceinline__ void update_odd(const Domain<R>& d, S* __restrict__ f,
+                                                    const R* F, const uint32_t* key, int i, int x,
+                                                    int y, int z, bool bulk_yz, bool bulk_x) {
+  if (SOLIDS && d.solid) {
+    // a warp with any solid-touching link takes the full addressing with
+    // the cells' solid bits (the vote comes before any lane leaves)
+    const uint32_t sm = d.solid[i];
+    if (warp_any(sm != 0u)) {
+      if (sm & kSolidCell) return;
+      // In the bulk only the solid bits redirect a link: one select between
+      // two tabled offsets, or the x-only addressing, instead of the full
+      // one (porous 192^3, 30 % solid, D3Q18 FP32: 153 us a step before, 141
+      // now).
+      if (!d.sym && bulk_yz) {
+        if (bulk_x) {
+          Links L = make_links_interior(d);
+          L.solid = sm;
+          update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
+        } else {
+          Links L = make_links_x(d, x);
+          L.solid = sm;
+          update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
+        }
+        return;
+      }
+      if (d.sym)
+        update_with_links<Q, S, R, true, FORCE, SR, CG, true, true, WIDE>(
+            d, f, i, make_links(d, x, y, z), F, key);
+      else
+        update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(
+            d, f, i, make_links(d, x, y, z), F, key);
+      return;
+    }
+  }
+  if (bulk_yz) {
+    if (bulk_x)
+      update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(
+          d, f, i, make_links_interior(d), F, key);
+    else if (d.sym)
+      update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(
+          d, f, i, make_links_x(d, x), F, key);
+    else
+      update_with_links<Q, S, R, true, FORCE, SR, CG, false, false, WIDE>(
+          d, f, i, make_links_x(d, x), F, key);
+  } else if (d.sym) {
+    update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(
+        d, f, i, make_links(d, x, y, z), F, key);
+  } else {
+    update_with_links<Q, S, R, true, FORCE, SR, CG, false, false, WIDE>(
+        d, f, i, make_links(d, x, y, z), F, key);
+  }
+}
+
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,
           bool CG = false, bool WIDE = false, bool SOLIDS = true>
 __host__ __device__ __forceinline__ void update_cell_at(const Domain<R>& d, S* __restrict__ f,
                                                         const R* F, const uint32_t* key, int x,
                                                         int y, int z, int x_lo, int x_hi) {
   const int i = x + d.nx * (y + d.ny * z);
-  if constexpr (!ODD) {
-    if (SOLIDS && d.solid && (d.solid[i] & kSolidCell)) return;  // solid cells hold no flow
-    Links L{};
-    update_with_links<Q, S, R, false, FORCE, SR, CG, true, false, WIDE>(d, f, i, L, F, key);
-  } else {
-    if (SOLIDS && d.solid) {
-      // a warp with any solid-touching link takes the full addressing with
-      // the cells' solid bits (the vote comes before any lane leaves)
-      const uint32_t sm = d.solid[i];
-      if (warp_any(sm != 0u)) {
-        if (sm & kSolidCell) return;
-        // In the bulk only the solid bits redirect a link: one select between
-        // two tabled offsets, or the x-only addressing, instead of the full
-        // one (porous 192^3, 30 % solid, D3Q18 FP32: 153 us a step before, 141
-        // now).
-        if (!d.sym && y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
-          if (x_lo > 0 && x_hi < d.nx - 1) {
-            Links L = make_links_interior(d);
-            L.solid = sm;
-            update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
-          } else {
-            Links L = make_links_x(d, x);
-            L.solid = sm;
-            update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(d, f, i, L, F, key);
-          }
-          return;
-        }
-        if (d.sym)
-          update_with_links<Q, S, R, true, FORCE, SR, CG, true, true, WIDE>(
-              d, f, i, make_links(d, x, y, z), F, key);
-        else
-          update_with_links<Q, S, R, true, FORCE, SR, CG, false, true, WIDE>(
-              d, f, i, make_links(d, x, y, z), F, key);
-        return;
-      }
-    }
-    if (y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1) {
-      if (x_lo > 0 && x_hi < d.nx - 1)
-        update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(d, f, i, make_links_interior(d), F,
-                                                        key);
-      else if (d.sym)
-        update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(d, f, i, make_links_x(d, x), F,
-                                                              key);
-      else
-        update_with_links<Q, S, R, true, FORCE, SR, CG, false, false, WIDE>(d, f, i, make_links_x(d, x), F,
-                                                               key);
-    } else if (d.sym) {
-      update_with_links<Q, S, R, true, FORCE, SR, CG, true, false, WIDE>(d, f, i, make_links(d, x, y, z), F,
-                                                            key);
-    } else {
-      update_with_links<Q, S, R, true, FORCE, SR, CG, false, false, WIDE>(d, f, i, make_links(d, x, y, z), F,
-                                                             key);
-    }
-  }
+  if constexpr (!ODD)
+    update_even<Q, S, R, FORCE, SR, CG, WIDE, SOLIDS>(d, f, F, key, i);
+  else
+    update_odd<Q, S, R, FORCE, SR, CG, WIDE, SOLIDS>(
+        d, f, F, key, i, x, y, z, y > 0 && y < d.ny - 1 && z > 0 && z < d.nz - 1,
+        x_lo > 0 && x_hi < d.nx - 1);
 }
 
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,

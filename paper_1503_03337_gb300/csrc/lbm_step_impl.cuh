@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cmath>
+#include <type_traits>
 
 #include "lbm_internal.h"
 #include "lbm_kernels.cuh"
@@ -28,11 +29,17 @@ constexpr int step_min_blocks() {
   return sizeof(S) == 8 ? 2 : 4;
 }
 
-// WIDE: 64-bit population offsets, for domains with Q*N >= 2^31.
-template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR, bool WIDE = false>
-__global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Domain<R> d) {
-  pdl_release();
+// Cells by rows: nx a multiple of 32, or a small box (steps_in_line).
+// WIDE: 64-bit population offsets, for domains with Q*N >= 2^31.  SOLIDS =
+// false: d has no solid mask (odd steps then carry five addressing variants
+// instead of nine).  The next launch is let in after the wait, not before it:
+// a trigger before it makes several later grids resident, whose blocks take
+// whatever slots are free and bunch on some SMs (33^3 D3Q14 FP32: 3.07 us a
+// step with the trigger first, 2.87 so; boxes of many waves do not change).
+template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool WIDE, bool SOLIDS>
+__global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Domain<float> d) {
   pdl_acquire();
+  pdl_release();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = slab_plane(d);
@@ -41,8 +48,47 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
   // blockDim.x is a multiple of 32 (then the path choice is warp-uniform)
   const int x_lo = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   const int x_hi = x_lo + 31;
-  update_cell<Q, S, R, ODD, FORCE, SR, false, WIDE>(d, static_cast<S*>(d.f), x, y, z, x_lo,
-                                                    x_hi);
+  update_cell<Q, S, float, ODD, FORCE, SR, false, WIDE, SOLIDS>(d, static_cast<S*>(d.f), x, y, z,
+                                                                x_lo, x_hi);
+}
+
+// The cells of a launch in linear order (k_step_line).
+struct LineArgs {
+  int first, cells;  // cells first .. first + cells - 1, past N going on at 0
+  FastDiv by_x, by_y;
+};
+
+// One cell per thread, cells in linear order whatever row they are in, so that
+// no lanes are left empty at the ends of rows; the warp votes on the
+// addressing variant.  The step is bound by instruction issue in L2-sized
+// boxes and with 2-byte storage, so what it gains is the padding: us a step by
+// rows and so, 97x97x49 D3Q18 FP32 10.8 and 9.6, 65^3 8.4 and 6.8, 129^3 47.2
+// and 41.8, 200^3 154 and 146, 97^3 FP16 17.2 and 13.6, 161^3 FP16 75.9 and
+// 67.4, 100^3 D3Q26 FP16 34.8 and 23.9.  The coordinates of a cell are formed
+// before the wait for the previous step.  SOLIDS: d has a solid mask; every
+// such box runs here (100^3, 30 % solid, FP32: 20.9 and 17.8; 192^3, whose rows
+// have no padding, 137.7 and 137.0), so k_step carries no solid code.
+template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool SOLIDS>
+__global__ void __launch_bounds__(256, step_min_blocks<Q, S>()) k_step_line(Domain<float> d,
+                                                                            LineArgs a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= a.cells) return;
+  unsigned u = (unsigned)a.first + (unsigned)t;
+  const int i = (int)(u < (unsigned)d.N ? u : u - (unsigned)d.N);
+  S* const f = static_cast<S*>(d.f);
+  if constexpr (!ODD) {
+    pdl_acquire();
+    pdl_release();
+    update_even<Q, S, float, FORCE, SR, false, false, SOLIDS>(d, f, d.F, &d.key, i);
+  } else {
+    const int r = a.by_x(i), z = a.by_y(r), x = i - r * d.nx, y = r - z * d.ny;
+    const bool yz = y == 0 || y == d.ny - 1 || z == 0 || z == d.nz - 1;
+    const bool bulk_yz = !warp_any(yz), bulk_x = !warp_any(x == 0 || x == d.nx - 1);
+    pdl_acquire();
+    pdl_release();
+    update_odd<Q, S, float, FORCE, SR, false, false, SOLIDS>(d, f, d.F, &d.key, i, x, y, z,
+                                                             bulk_yz, bulk_x);
+  }
 }
 
 // FP64 storage: cells in linear order, one after another whatever row they
@@ -55,6 +101,8 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
 // 16x16x32 D3Q18: 30.8 us a step with 32 x 8 blocks of rows, 8.2 so.
 template <int Q, bool ODD, bool FORCE, bool WIDE>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(Domain<double> d) {
+  // before the wait: with so many small blocks a late trigger costs more than
+  // the even spread gains (16x16x32 D3Q18: 8.2 us a step so, 9.2 after it)
   pdl_release();
   pdl_acquire();
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // N < 2^31
@@ -87,8 +135,8 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(
 // for Q14).
 template <int Q, typename S, bool FORCE, bool SR>
 __global__ void __launch_bounds__(256, 3) k_step_pair(Domain<float> d) {
-  pdl_release();
   pdl_acquire();
+  pdl_release();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = slab_plane(d);
@@ -118,75 +166,108 @@ void launch_f64(const Domain<double>& d, bool odd, bool force, bool wide, const 
              b.pdl != 0, st);
 }
 
-template <int Q, typename S, typename R, bool SR>
-void launch_parity(const Domain<R>& d, bool odd, bool force, bool wide, dim3 grid, dim3 block,
+// fn.operator()<ODD, FORCE>() for the two run-time flags.
+template <typename Fn>
+void by_flags(bool odd, bool force, Fn&& fn) {
+  if (odd) {
+    if (force) fn.template operator()<true, true>();
+    else fn.template operator()<true, false>();
+  } else {
+    if (force) fn.template operator()<false, true>();
+    else fn.template operator()<false, false>();
+  }
+}
+
+template <int Q, typename S, bool SR>
+void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int planes,
                    const BlockShape& b, cudaStream_t st) {
+  const bool pdl = b.pdl != 0;
+  const dim3 block(b.bx, b.by);
+  const int by = (d.ny + b.by - 1) / b.by;
+  const dim3 grid((d.nx + b.bx - 1) / b.bx, by, planes);
   // Q*N >= 2^31: one cell per thread with 64-bit population offsets
   if (wide) {
-    if (odd) {
-      if (force) launch_one(k_step<Q, S, R, true, true, SR, true>, d, grid, block, b.pdl != 0, st);
-      else launch_one(k_step<Q, S, R, true, false, SR, true>, d, grid, block, b.pdl != 0, st);
-    } else {
-      if (force) launch_one(k_step<Q, S, R, false, true, SR, true>, d, grid, block, b.pdl != 0, st);
-      else launch_one(k_step<Q, S, R, false, false, SR, true>, d, grid, block, b.pdl != 0, st);
-    }
+    by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
+      launch_one(k_step<Q, S, ODD, FORCE, SR, true, true>, d, grid, block, pdl, st);
+    });
     return;
   }
   // two cells per thread: even steps of FP32 / FP16 / BF16 storage with nx
   // even and no solid nodes, Q = 14 or 18 (the 52 packed values of a Q = 26
   // pair would not fit the registers); every other step runs one cell per
   // thread
-  if constexpr (sizeof(S) <= 4 && Q != 26) {
+  if constexpr (Q != 26) {
     if (b.cpt == 2 && !odd && d.nx % 2 == 0 && !d.solid) {
-      grid.x = (d.nx / 2 + block.x - 1) / block.x;
-      if (force) launch_one(k_step_pair<Q, S, true, SR>, d, grid, block, b.pdl != 0, st);
-      else launch_one(k_step_pair<Q, S, false, SR>, d, grid, block, b.pdl != 0, st);
+      const dim3 half((d.nx / 2 + b.bx - 1) / b.bx, by, planes);
+      if (force) launch_one(k_step_pair<Q, S, true, SR>, d, half, block, pdl, st);
+      else launch_one(k_step_pair<Q, S, false, SR>, d, half, block, pdl, st);
       return;
     }
   }
-  if (odd) {
-    if (force) launch_one(k_step<Q, S, R, true, true, SR>, d, grid, block, b.pdl != 0, st);
-    else launch_one(k_step<Q, S, R, true, false, SR>, d, grid, block, b.pdl != 0, st);
-  } else {
-    if (force) launch_one(k_step<Q, S, R, false, true, SR>, d, grid, block, b.pdl != 0, st);
-    else launch_one(k_step<Q, S, R, false, false, SR>, d, grid, block, b.pdl != 0, st);
+  if (d.solid || steps_in_line(d.nx, d.ny, d.N)) {
+    const int plane = d.nx * d.ny, cells = planes * plane;
+    const unsigned threads = b.bx * b.by;
+    const LineArgs a{d.z0 * plane, cells, FastDiv(d.nx), FastDiv(d.ny)};
+    const dim3 blocks(((unsigned)cells + threads - 1) / threads);
+    by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
+      launch_pdl(d.solid ? k_step_line<Q, S, ODD, FORCE, SR, true>
+                         : k_step_line<Q, S, ODD, FORCE, SR, false>,
+                 blocks, dim3(threads), pdl, st, d, a);
+    });
+    return;
   }
+  by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
+    launch_one(k_step<Q, S, ODD, FORCE, SR, false, false>, d, grid, block, pdl, st);
+  });
 }
 
 // Steps n .. n + count - 1, slab by slab (run_slabs).  The descriptor is
 // built once; a launch changes only its planes, force and rounding key, so it
 // costs the host 1.8 us where rebuilding the descriptor made it 5.5 us (16^3
 // D3Q18 FP32: 6.0 us a step before, 2.0 us now).
-template <int Q, typename S, typename R>
+template <int Q, typename S, bool SR>
 cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockShape b,
                          const SlabPlan& plan, cudaStream_t st) {
+  using R = std::conditional_t<sizeof(S) == 8, double, float>;
   const double zero[3] = {0.0, 0.0, 0.0};
   // the force-carrying update whenever the amplitude is nonzero (also at the
   // steps where a periodic force passes through zero), as the batch does
   const bool force = dd.force[0] != 0.0 || dd.force[1] != 0.0 || dd.force[2] != 0.0;
   Domain<R> d = to_domain<R>(dd, zero);
-  const dim3 block(b.bx, b.by, 1);
   const bool wide = (int64_t)dd.Q * dd.N >= (int64_t(1) << 31);
-  bool sr = false;
-  if constexpr (Stochastic<S>::enabled) sr = dd.rounding == LBM_ROUND_STOCHASTIC;
   return run_slabs(dd.nz, dd.per[2] != 0, plan, count, [&](int64_t s, int z0, int planes) {
     double F[3];
     force_at(dd, n + s, F);
     for (int c = 0; c < 3; ++c) d.F[c] = R(F[c]);
     d.key = step_key(n + s);
     d.z0 = z0;
-    const dim3 grid((dd.nx + b.bx - 1) / b.bx, (dd.ny + b.by - 1) / b.by, planes);
     const bool odd = ((n + s) & 1) != 0;
-    if constexpr (sizeof(S) == 8) {
-      launch_f64<Q>(d, odd, force, wide, b, st);
-    } else {
-      if constexpr (Stochastic<S>::enabled) {
-        if (sr) launch_parity<Q, S, R, true>(d, odd, force, wide, grid, block, b, st);
-      }
-      if (!sr) launch_parity<Q, S, R, false>(d, odd, force, wide, grid, block, b, st);
-    }
+    if constexpr (sizeof(S) == 8) launch_f64<Q>(d, odd, force, wide, b, st);
+    else launch_parity<Q, S, SR>(d, odd, force, wide, planes, b, st);
     return cudaGetLastError();
   });
+}
+
+#define LBM_STEP_UNIT(Q, S, SR)                                                              \
+  template cudaError_t launch_typed<Q, S, SR>(const DomainDesc&, int64_t, int64_t, BlockShape, \
+                                              const SlabPlan&, cudaStream_t)
+#define LBM_STEP_EXTERN(Q, S, SR) extern LBM_STEP_UNIT(Q, S, SR)
+
+template <int Q>
+cudaError_t launch_storage(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
+                           const SlabPlan& plan, cudaStream_t st) {
+  const bool sr = d.rounding == LBM_ROUND_STOCHASTIC;
+  switch (d.storage) {
+    case LBM_STORAGE_F64: return launch_typed<Q, double, false>(d, n, count, b, plan, st);
+    case LBM_STORAGE_F32: return launch_typed<Q, float, false>(d, n, count, b, plan, st);
+    case LBM_STORAGE_F16:
+      return sr ? launch_typed<Q, __half, true>(d, n, count, b, plan, st)
+                : launch_typed<Q, __half, false>(d, n, count, b, plan, st);
+    case LBM_STORAGE_BF16:
+      return sr ? launch_typed<Q, __nv_bfloat16, true>(d, n, count, b, plan, st)
+                : launch_typed<Q, __nv_bfloat16, false>(d, n, count, b, plan, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace lbm

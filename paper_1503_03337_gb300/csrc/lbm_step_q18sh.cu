@@ -1,0 +1,8 @@
+// Step kernels for Q = 18, FP16 storage, stochastic rounding (see lbm_step_impl.cuh).
+#include "lbm_step_impl.cuh"
+
+namespace lbm {
+
+LBM_STEP_UNIT(18, __half, true);
+
+}  // namespace lbm

@@ -1,22 +1,19 @@
-// Step kernels for Q = 26 with FP64 and FP32 storage (see lbm_step_impl.cuh);
-// the 2-byte storage types are in lbm_step_q26h.cu, so the two compile in
-// parallel.
+// Dispatch of the Q = 26 steps by storage type and rounding, and the FP32 step
+// kernels (see lbm_step_impl.cuh); every other type has a unit of its own, so
+// that they compile in parallel.
 #include "lbm_step_impl.cuh"
 
 namespace lbm {
 
-cudaError_t launch_step_q26_half(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                                 const SlabPlan& plan, cudaStream_t st);
+LBM_STEP_EXTERN(26, double, false);
+LBM_STEP_EXTERN(26, __half, false);
+LBM_STEP_EXTERN(26, __half, true);
+LBM_STEP_EXTERN(26, __nv_bfloat16, false);
+LBM_STEP_EXTERN(26, __nv_bfloat16, true);
 
 cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
                             const SlabPlan& plan, cudaStream_t st) {
-  switch (d.storage) {
-    case LBM_STORAGE_F64: return launch_typed<26, double, double>(d, n, count, b, plan, st);
-    case LBM_STORAGE_F32: return launch_typed<26, float, float>(d, n, count, b, plan, st);
-    case LBM_STORAGE_F16:
-    case LBM_STORAGE_BF16: return launch_step_q26_half(d, n, count, b, plan, st);
-  }
-  return cudaErrorInvalidValue;
+  return launch_storage<26>(d, n, count, b, plan, st);
 }
 
 }  // namespace lbm

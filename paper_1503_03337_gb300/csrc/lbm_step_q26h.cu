@@ -1,16 +1,8 @@
-// Step kernels for Q = 26 with FP16 storage (see lbm_step_impl.cuh); BF16 is
-// in lbm_step_q26b.cu, so the two compile in parallel.
+// Step kernels for Q = 26, FP16 storage, rounding to nearest (see lbm_step_impl.cuh).
 #include "lbm_step_impl.cuh"
 
 namespace lbm {
 
-cudaError_t launch_step_q26_bf16(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                                 const SlabPlan& plan, cudaStream_t st);
-
-cudaError_t launch_step_q26_half(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                                 const SlabPlan& plan, cudaStream_t st) {
-  if (d.storage == LBM_STORAGE_F16) return launch_typed<26, __half, float>(d, n, count, b, plan, st);
-  return launch_step_q26_bf16(d, n, count, b, plan, st);
-}
+LBM_STEP_UNIT(26, __half, false);
 
 }  // namespace lbm

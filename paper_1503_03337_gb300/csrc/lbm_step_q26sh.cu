@@ -1,0 +1,8 @@
+// Step kernels for Q = 26, FP16 storage, stochastic rounding (see lbm_step_impl.cuh).
+#include "lbm_step_impl.cuh"
+
+namespace lbm {
+
+LBM_STEP_UNIT(26, __half, true);
+
+}  // namespace lbm
