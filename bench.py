@@ -198,7 +198,7 @@ def step_launches(Q, storage, n, updates, l2_bytes):
     rule of slab_plan and run_slabs)."""
     plane = n * n * Q * 4
     touched = min(l2_bytes * 62 // 100 // plane, n)
-    if storage != "f32" or plane * n * 100 < l2_bytes * 65 or touched < 10:
+    if storage != "f32" or plane * n * 100 < l2_bytes * 65 or touched < (18 if Q == 26 else 10):
         return updates
     depth = min(16, touched * 3 // 8)
     slabs = -(-(n - depth) // (touched - depth))
