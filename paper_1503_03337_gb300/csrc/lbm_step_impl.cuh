@@ -216,8 +216,11 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
     });
     return;
   }
+  // the build of the D3Q18 BF16 stochastic step that carries the solid code is
+  // scheduled better: 244 against 250 us at 256^3 (D3Q14 210 against 200)
+  constexpr bool kSolids = Q == 18 && SR && std::is_same_v<S, __nv_bfloat16>;
   by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
-    launch_one(k_step<Q, S, ODD, FORCE, SR, false, false>, d, grid, block, pdl, st);
+    launch_one(k_step<Q, S, ODD, FORCE, SR, false, kSolids>, d, grid, block, pdl, st);
   });
 }
 
