@@ -190,7 +190,7 @@ int lbm_create(const lbm_desc* desc, void* cuda_stream, lbm_handle** out) {
   h->d.nz = desc->nz;
   h->d.storage = desc->storage;
   h->d.N = N;
-  h->block = default_block(desc->nx, desc->ny, N, desc->storage);
+  h->block = default_block(desc->Q, desc->nx, desc->ny, N, desc->storage);
 
   const size_t fbytes = (size_t)N * desc->Q * b;
   e = cudaMalloc(&h->d.f, fbytes);
@@ -623,7 +623,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
     b.pdl = h->block.pdl;
     if (b.bx * b.cpt > xmax && b.bx > 32) continue;
     if (b.cpt == 2 && (h->d.storage == LBM_STORAGE_F64 || h->d.Q == 26 ||
-                       (int64_t)h->d.Q * h->d.N >= (int64_t(1) << 31)))
+                       wide_offsets(h->d.Q, h->d.N)))
       continue;
     int64_t n = n0;
     if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, plan, h->stream);

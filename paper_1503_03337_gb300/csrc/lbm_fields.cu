@@ -526,7 +526,7 @@ cudaError_t launch_reduce(const DomainDesc& dd, int64_t n, double* u_prev, int h
       const PairSum f0 = pair_of(0.5 * F[0]), f1 = pair_of(0.5 * F[1]),
                     f2 = pair_of(0.5 * F[2]);
       const PairSum pr = pair_of(3.0 * (1.0 - Lattice<Q>::w0) * dd.p_ref);
-      const bool wide = (int64_t)dd.Q * dd.N >= (int64_t(1) << 31);
+      const bool wide = wide_offsets(dd.Q, dd.N);
       auto kernel = wide ? (odd ? k_reduce_pair<Q, S, true, true> : k_reduce_pair<Q, S, false, true>)
                          : (odd ? k_reduce_pair<Q, S, true, false> : k_reduce_pair<Q, S, false, false>);
       kernel<<<(int)g, kReduceThreads, 0, st>>>(df, a, f0, f1, f2, pr);

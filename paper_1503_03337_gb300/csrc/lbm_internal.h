@@ -63,10 +63,13 @@ struct FastDiv {
   }
 };
 
+// Q * N >= 2^31: 64-bit population offsets.
+inline bool wide_offsets(int Q, int64_t N) { return Q * N >= (int64_t(1) << 31); }
+
 // The default launch of a box; 4- and 2-byte storage runs its cells in linear
 // order (k_step_line) or by rows (k_step).
-BlockShape default_block(int nx, int ny, int64_t N, int storage);
-bool steps_in_line(int nx, int ny, int64_t N);
+BlockShape default_block(int Q, int nx, int ny, int64_t N, int storage);
+bool steps_in_line(int Q, int nx, int ny, int64_t N);
 
 // The face fields of d (per, moving, sym, neq_*, uw) from a geometry.
 // Returns nullptr, or the reason the geometry is invalid (then d is

@@ -130,13 +130,15 @@ SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
 // 4.6, 45^3 FP16 (91) 4.3 and 4.3, 49^3 (118) 5.1 and 4.6, 65^3 8.4 and 6.8.
 // Blocks of four warps: 65^3 6.96 us with eight, 6.75 with four, 7.07 with
 // two; 97^3 FP16 14.0, 13.6 and 16.5; 100^3 D3Q26 FP16 27.3, 23.9 and 24.6.
-bool steps_in_line(int nx, int ny, int64_t N) {
-  return nx % 32 != 0 && nx > 1 && ny > 1 && N >= 100000;
+// Boxes with 64-bit population offsets go by rows, so they keep the row shape
+// below: with one row a block, ny > 65535 would exceed the grid's y limit.
+bool steps_in_line(int Q, int nx, int ny, int64_t N) {
+  return nx % 32 != 0 && nx > 1 && ny > 1 && N >= 100000 && !wide_offsets(Q, N);
 }
 
-BlockShape default_block(int nx, int ny, int64_t N, int storage) {
+BlockShape default_block(int Q, int nx, int ny, int64_t N, int storage) {
   if (storage == LBM_STORAGE_F64) return {32, 1, 1};  // one warp each (k_step_f64)
-  if (steps_in_line(nx, ny, N)) return {128, 1, 1};
+  if (steps_in_line(Q, nx, ny, N)) return {128, 1, 1};
   int bx = 32;
   while (bx < nx && bx < 128) bx *= 2;
   int by = 256 / bx;

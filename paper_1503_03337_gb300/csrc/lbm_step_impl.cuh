@@ -204,7 +204,7 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
       return;
     }
   }
-  if (d.solid || steps_in_line(d.nx, d.ny, d.N)) {
+  if (d.solid || steps_in_line(Q, d.nx, d.ny, d.N)) {
     const int plane = d.nx * d.ny, cells = planes * plane;
     const unsigned threads = b.bx * b.by;
     const LineArgs a{d.z0 * plane, cells, FastDiv(d.nx), FastDiv(d.ny)};
@@ -237,7 +237,7 @@ cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockSh
   // steps where a periodic force passes through zero), as the batch does
   const bool force = dd.force[0] != 0.0 || dd.force[1] != 0.0 || dd.force[2] != 0.0;
   Domain<R> d = to_domain<R>(dd, zero);
-  const bool wide = (int64_t)dd.Q * dd.N >= (int64_t(1) << 31);
+  const bool wide = wide_offsets(dd.Q, dd.N);
   return run_slabs(dd.nz, dd.per[2] != 0, plan, count, [&](int64_t s, int z0, int planes) {
     double F[3];
     force_at(dd, n + s, F);
