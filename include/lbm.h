@@ -234,7 +234,10 @@ int lbm_init_equilibrium(lbm_handle *h, const double *u, const double *p, int on
 /* Queue nsteps fused steps (stream + collide, Eq. mrteqvT) on the stream.
  * Asynchronous.  Returns LBM_EUNSTABLE without queuing anything if an
  * earlier reduction found non-finite values (until the next init or
- * write_populations). */
+ * write_populations).  If a launch fails, the step counter names the last
+ * step that was queued whole; where the failure leaves parts of the box at
+ * different steps, stepping, reading, reducing and autotuning return
+ * LBM_ECUDA until the next init or write_populations. */
 int lbm_step(lbm_handle *h, int64_t nsteps);
 
 /* Current step counter n (populations hold f^n). */

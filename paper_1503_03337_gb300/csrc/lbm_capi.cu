@@ -21,6 +21,7 @@ struct lbm_handle {
   lbm_geom geom{};
   lbm_params params{};
   int64_t n = 0;
+  bool torn = false;            // a failed lbm_step left planes at different steps
   BlockShape block{32, 8, 1};
   // reductions
   double* u_prev = nullptr;     // 3*N snapshot, allocated on first use
@@ -133,6 +134,15 @@ int apply_geometry(lbm_handle* h, const lbm_geom* g) {
 
 int check(lbm_handle* h) {
   if (!h) return fail(LBM_EINVAL, "null handle");
+  return LBM_OK;
+}
+
+// check, and the populations belong to one step.
+int check_state(lbm_handle* h) {
+  if (int rc = check(h)) return rc;
+  if (h->torn)
+    return fail(LBM_ECUDA, "an earlier lbm_step failed part-way through the box: "
+                           "initialise or write the populations first");
   return LBM_OK;
 }
 
@@ -359,6 +369,7 @@ int lbm_init_equilibrium(lbm_handle* h, const double* u, const double* p, int on
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "init synchronize");
   h->n = 0;
+  h->torn = false;
   h->have_prev = 0;
   h->prev_step = -1;
   h->stats_step = -1;
@@ -387,7 +398,7 @@ static int run_reduction(lbm_handle* h) {
 }
 
 int lbm_step(lbm_handle* h, int64_t nsteps) {
-  if (int rc = check(h)) return rc;
+  if (int rc = check_state(h)) return rc;
   if (nsteps < 0) return fail(LBM_EINVAL, "nsteps < 0");
   if (static_cast<volatile double*>(h->stats_host)[kNumSums - 1] > 0.0)
     return fail(LBM_EUNSTABLE, "a reduction found non-finite values");
@@ -399,9 +410,11 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     // up to the next boundary pass or reduction
     int64_t m = neq ? 1 : nsteps;
     if (K > 0) m = std::min<int64_t>(m, K - h->n % K);
-    cudaError_t e = launch_steps(h->d, h->n, m, h->block, plan, h->stream);
+    StepProgress done;
+    cudaError_t e = launch_steps(h->d, h->n, m, h->block, plan, h->stream, &done);
+    h->n += done.steps;
+    h->torn = done.torn;
     if (e != cudaSuccess) return cuda_fail(e, "step kernel");
-    h->n += m;
     nsteps -= m;
     if (neq) {  // the extrapolation boundaries of the new time level
       e = launch_neq(h->d, h->n, h->block.pdl != 0, h->stream);
@@ -434,7 +447,7 @@ int lbm_set_step(lbm_handle* h, int64_t n) {
 }
 
 int lbm_read_fields(lbm_handle* h, unsigned mask, void* dst, int dst_on_device, int dtype) {
-  if (int rc = check(h)) return rc;
+  if (int rc = check_state(h)) return rc;
   if (!dst) return fail(LBM_EINVAL, "null destination");
   if (mask == 0 || (mask & ~7u)) return fail(LBM_EINVAL, "bad field mask");
   if (dtype != LBM_DTYPE_F64 && dtype != LBM_DTYPE_F32) return fail(LBM_EINVAL, "bad dtype");
@@ -472,6 +485,7 @@ int lbm_write_populations(lbm_handle* h, const double* src, int src_on_device) {
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (!rc && e != cudaSuccess) rc = cuda_fail(e, "write synchronize");
   if (!rc) {
+    h->torn = false;
     h->stats_host[kNumSums - 1] = 0.0;
     h->have_prev = 0;
     h->prev_step = -1;
@@ -496,7 +510,7 @@ static void fill_stats(lbm_handle* h, lbm_stats* out) {
 }
 
 int lbm_reductions(lbm_handle* h, lbm_stats* out) {
-  if (int rc = check(h)) return rc;
+  if (int rc = check_state(h)) return rc;
   if (!out) return fail(LBM_EINVAL, "null output");
   DeviceGuard dg(h->device);
   if (int rc = run_reduction(h)) return rc;
@@ -584,7 +598,7 @@ const BlockShape kCandidates[] = {{32, 1, 1},  {32, 2, 1}, {32, 4, 1}, {32, 8, 1
 }  // namespace
 
 int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) {
-  if (int rc = check(h)) return rc;
+  if (int rc = check_state(h)) return rc;
   DeviceGuard dg(h->device);
   const auto key =
       std::make_tuple(h->d.Q, h->d.storage, h->d.rounding, h->d.nx, h->d.ny, h->d.nz);
@@ -626,10 +640,10 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
                        wide_offsets(h->d.Q, h->d.N)))
       continue;
     int64_t n = n0;
-    if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, plan, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, plan, h->stream, nullptr);
     n += 2;
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    if (e == cudaSuccess) e = launch_steps(h->d, n, trials, b, plan, h->stream);
+    if (e == cudaSuccess) e = launch_steps(h->d, n, trials, b, plan, h->stream, nullptr);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float t = 0.f;

@@ -112,9 +112,18 @@ struct SlabPlan {
 // The slabs of d's steps on a device with l2_bytes of L2.
 SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes);
 
-// launch(s, z0, planes) for every step s of 0 .. count - 1 and slab.
+// What was queued of a run of steps: `steps` of the whole box, and, if torn,
+// some planes further on (a launch failed within a round of slabs).
+struct StepProgress {
+  int64_t steps = 0;
+  bool torn = false;
+};
+
+// launch(s, z0, planes) for every step s of 0 .. count - 1 and slab, up to the
+// first launch that fails; *done (if not null) tells how far it came.
 template <typename Fn>
-cudaError_t run_slabs(int nz, bool periodic, const SlabPlan& plan, int64_t count, Fn&& launch) {
+cudaError_t run_slabs(int nz, bool periodic, const SlabPlan& plan, int64_t count, Fn&& launch,
+                      StepProgress* done = nullptr) {
   // begin(k) leaves every slab the same number of planes per round: (planes
   // to share out) / slabs, plus the depth-wide ramp at the bottom
   const int64_t share = periodic ? nz : nz - plan.depth;
@@ -131,15 +140,20 @@ cudaError_t run_slabs(int nz, bool periodic, const SlabPlan& plan, int64_t count
           if (k == 0) lo = s;
           if (k == slabs - 1) hi = nz + s;
         }
-        if (cudaError_t e = launch(s0 + s, lo, hi - lo)) return e;
+        if (cudaError_t e = launch(s0 + s, lo, hi - lo)) {
+          if (done) *done = slabs == 1 ? StepProgress{s0 + s, false}
+                                       : StepProgress{s0, k > 0 || s > 0};
+          return e;
+        }
       }
   }
+  if (done) *done = {count, false};
   return cudaSuccess;
 }
 
 // Queue the fused steps n .. n + count - 1 (parity of each its number's).
 cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                         const SlabPlan& plan, cudaStream_t st);
+                         const SlabPlan& plan, cudaStream_t st, StepProgress* done);
 
 // f = f_eq(p - p_ref, u) at every node, stored for step 0 (even layout).
 cudaError_t launch_init(const DomainDesc& d, const double* u, const double* p,

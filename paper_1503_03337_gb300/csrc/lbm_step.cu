@@ -147,18 +147,18 @@ BlockShape default_block(int Q, int nx, int ny, int64_t N, int storage) {
 }
 
 cudaError_t launch_step_q14(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            const SlabPlan& plan, cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st, StepProgress* done);
 cudaError_t launch_step_q18(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            const SlabPlan& plan, cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st, StepProgress* done);
 cudaError_t launch_step_q26(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            const SlabPlan& plan, cudaStream_t st);
+                            const SlabPlan& plan, cudaStream_t st, StepProgress* done);
 
 cudaError_t launch_steps(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                         const SlabPlan& plan, cudaStream_t st) {
+                         const SlabPlan& plan, cudaStream_t st, StepProgress* done) {
   if (d.N == 0) return cudaSuccess;
-  if (d.Q == 14) return launch_step_q14(d, n, count, b, plan, st);
-  if (d.Q == 18) return launch_step_q18(d, n, count, b, plan, st);
-  if (d.Q == 26) return launch_step_q26(d, n, count, b, plan, st);
+  if (d.Q == 14) return launch_step_q14(d, n, count, b, plan, st, done);
+  if (d.Q == 18) return launch_step_q18(d, n, count, b, plan, st, done);
+  if (d.Q == 26) return launch_step_q26(d, n, count, b, plan, st, done);
   return cudaErrorInvalidValue;
 }
 

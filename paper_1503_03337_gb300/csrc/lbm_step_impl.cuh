@@ -230,7 +230,7 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
 // D3Q18 FP32: 6.0 us a step before, 2.0 us now).
 template <int Q, typename S, bool SR>
 cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockShape b,
-                         const SlabPlan& plan, cudaStream_t st) {
+                         const SlabPlan& plan, cudaStream_t st, StepProgress* done) {
   using R = std::conditional_t<sizeof(S) == 8, double, float>;
   const double zero[3] = {0.0, 0.0, 0.0};
   // the force-carrying update whenever the amplitude is nonzero (also at the
@@ -248,27 +248,27 @@ cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockSh
     if constexpr (sizeof(S) == 8) launch_f64<Q>(d, odd, force, wide, b, st);
     else launch_parity<Q, S, SR>(d, odd, force, wide, planes, b, st);
     return cudaGetLastError();
-  });
+  }, done);
 }
 
 #define LBM_STEP_UNIT(Q, S, SR)                                                              \
   template cudaError_t launch_typed<Q, S, SR>(const DomainDesc&, int64_t, int64_t, BlockShape, \
-                                              const SlabPlan&, cudaStream_t)
+                                              const SlabPlan&, cudaStream_t, StepProgress*)
 #define LBM_STEP_EXTERN(Q, S, SR) extern LBM_STEP_UNIT(Q, S, SR)
 
 template <int Q>
 cudaError_t launch_storage(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                           const SlabPlan& plan, cudaStream_t st) {
+                           const SlabPlan& plan, cudaStream_t st, StepProgress* done) {
   const bool sr = d.rounding == LBM_ROUND_STOCHASTIC;
   switch (d.storage) {
-    case LBM_STORAGE_F64: return launch_typed<Q, double, false>(d, n, count, b, plan, st);
-    case LBM_STORAGE_F32: return launch_typed<Q, float, false>(d, n, count, b, plan, st);
+    case LBM_STORAGE_F64: return launch_typed<Q, double, false>(d, n, count, b, plan, st, done);
+    case LBM_STORAGE_F32: return launch_typed<Q, float, false>(d, n, count, b, plan, st, done);
     case LBM_STORAGE_F16:
-      return sr ? launch_typed<Q, __half, true>(d, n, count, b, plan, st)
-                : launch_typed<Q, __half, false>(d, n, count, b, plan, st);
+      return sr ? launch_typed<Q, __half, true>(d, n, count, b, plan, st, done)
+                : launch_typed<Q, __half, false>(d, n, count, b, plan, st, done);
     case LBM_STORAGE_BF16:
-      return sr ? launch_typed<Q, __nv_bfloat16, true>(d, n, count, b, plan, st)
-                : launch_typed<Q, __nv_bfloat16, false>(d, n, count, b, plan, st);
+      return sr ? launch_typed<Q, __nv_bfloat16, true>(d, n, count, b, plan, st, done)
+                : launch_typed<Q, __nv_bfloat16, false>(d, n, count, b, plan, st, done);
   }
   return cudaErrorInvalidValue;
 }

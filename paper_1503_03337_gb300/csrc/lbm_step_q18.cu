@@ -12,8 +12,8 @@ LBM_STEP_EXTERN(18, __nv_bfloat16, false);
 LBM_STEP_EXTERN(18, __nv_bfloat16, true);
 
 cudaError_t launch_step_q18(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,
-                            const SlabPlan& plan, cudaStream_t st) {
-  return launch_storage<18>(d, n, count, b, plan, st);
+                            const SlabPlan& plan, cudaStream_t st, StepProgress* done) {
+  return launch_storage<18>(d, n, count, b, plan, st, done);
 }
 
 }  // namespace lbm

@@ -7,9 +7,10 @@
 
 namespace lbm {
 // the rules launch nothing
-#define NO_LAUNCH(name)                                                                       \
-  cudaError_t name(const DomainDesc&, int64_t, int64_t, BlockShape, const SlabPlan&, cudaStream_t) { \
-    return cudaSuccess;                                                                       \
+#define NO_LAUNCH(name)                                                                         \
+  cudaError_t name(const DomainDesc&, int64_t, int64_t, BlockShape, const SlabPlan&, cudaStream_t, \
+                   StepProgress*) {                                                             \
+    return cudaSuccess;                                                                         \
   }
 NO_LAUNCH(launch_step_q14)
 NO_LAUNCH(launch_step_q18)
