@@ -329,12 +329,14 @@ int lbm_get_launch(lbm_handle *h, lbm_launch *launch);
 int lbm_set_overlap(lbm_handle *h, int32_t enable);
 
 /* Autotuner: time the step kernel on this domain for each candidate launch
- * shape (block shape, cells per thread; `trials` steps each, CUDA events on
- * the handle's stream) and keep the fastest.  The populations and step
+ * shape (block shape, cells per thread; `trials` steps each, rounded up to
+ * whole rounds where lbm_step sweeps the box in slabs; CUDA events on the
+ * handle's stream) and keep the fastest.  The populations and step
  * counter are saved before and restored after, so the state is unaffected
  * (the chosen cells per thread sets the FP32 rounding pattern, see
  * lbm_set_launch); the choice is cached per (Q, storage, rounding, nx, ny,
- * nz) for later handles of the same shape.  trials <= 0
+ * nz, with or without solid nodes, slabs) for later handles of the same
+ * shape.  trials <= 0
  * uses the cache only (or 8 trials on a miss).  Outputs may be NULL.
  * Synchronises; needs Q*N storage values of temporary device memory. */
 int lbm_autotune(lbm_handle *h, int32_t trials, lbm_launch *chosen, double *ms_per_step);

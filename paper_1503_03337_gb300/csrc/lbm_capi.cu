@@ -8,7 +8,6 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <tuple>
 
 #include "lbm_internal.h"
 
@@ -589,7 +588,7 @@ int lbm_set_overlap(lbm_handle* h, int32_t enable) {
 
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, int>, std::pair<BlockShape, double>> g_tune_cache;
+std::map<TuneKey, std::pair<BlockShape, double>> g_tune_cache;
 
 const BlockShape kCandidates[] = {{32, 1, 1},  {32, 2, 1}, {32, 4, 1}, {32, 8, 1},
                                   {64, 1, 1},  {64, 2, 1}, {64, 4, 1}, {128, 1, 1},
@@ -600,8 +599,8 @@ const BlockShape kCandidates[] = {{32, 1, 1},  {32, 2, 1}, {32, 4, 1}, {32, 8, 1
 int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) {
   if (int rc = check_state(h)) return rc;
   DeviceGuard dg(h->device);
-  const auto key =
-      std::make_tuple(h->d.Q, h->d.storage, h->d.rounding, h->d.nx, h->d.ny, h->d.nz);
+  const SlabPlan plan = slab_plan(h->d, h->l2_bytes);
+  const TuneKey key = tune_key(h->d, plan);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -613,8 +612,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
       return LBM_OK;
     }
   }
-  if (trials <= 0) trials = 8;
-  trials += trials & 1;  // even: equal numbers of even and odd steps
+  trials = tune_steps(trials > 0 ? trials : 8, plan);
   const size_t fbytes = (size_t)h->d.N * h->d.Q * storage_bytes(h->d.storage);
   void* saved = nullptr;
   cudaError_t e = cudaMalloc(&saved, fbytes);
@@ -630,15 +628,11 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
   BlockShape best = h->block;
   double best_ms = 1e300;
   const int64_t n0 = h->n;
-  const SlabPlan plan = slab_plan(h->d, h->l2_bytes);
-  const int xmax = ((h->d.nx + 31) / 32) * 32;
+  const bool kept = e == cudaSuccess;
   for (BlockShape b : kCandidates) {
     if (e != cudaSuccess) break;
     b.pdl = h->block.pdl;
-    if (b.bx * b.cpt > xmax && b.bx > 32) continue;
-    if (b.cpt == 2 && (h->d.storage == LBM_STORAGE_F64 || h->d.Q == 26 ||
-                       wide_offsets(h->d.Q, h->d.N)))
-      continue;
+    if (!tune_candidate(h->d, b)) continue;
     int64_t n = n0;
     if (e == cudaSuccess) e = launch_steps(h->d, n, 2, b, plan, h->stream, nullptr);
     n += 2;
@@ -656,7 +650,11 @@ int lbm_autotune(lbm_handle* h, int32_t trials, lbm_launch* chosen, double* ms) 
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(h->d.f, saved, fbytes, cudaMemcpyDeviceToDevice, h->stream);
   }
-  if (e != cudaSuccess) rc = cuda_fail(e, "autotune");
+  if (e != cudaSuccess) {
+    rc = cuda_fail(e, "autotune");
+    // a candidate that failed may have queued steps
+    if (kept) cudaMemcpyAsync(h->d.f, saved, fbytes, cudaMemcpyDeviceToDevice, h->stream);
+  }
   cudaError_t e2 = cudaStreamSynchronize(h->stream);
   if (!rc && e2 != cudaSuccess) rc = cuda_fail(e2, "autotune synchronize");
   if (e0) cudaEventDestroy(e0);

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <array>
 #include <cstdint>
 #include <string>
 
@@ -111,6 +112,15 @@ struct SlabPlan {
 
 // The slabs of d's steps on a device with l2_bytes of L2.
 SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes);
+
+// lbm_autotune: what its choice for a box depends on (the step kernels of the
+// box and the order they sweep it in), whether a block is a candidate of its
+// own there, and how many of at least `trials` steps it times: whole rounds of
+// slabs, as many even as odd steps.
+using TuneKey = std::array<int, 9>;
+TuneKey tune_key(const DomainDesc& d, const SlabPlan& plan);
+bool tune_candidate(const DomainDesc& d, const BlockShape& b);
+int tune_steps(int trials, const SlabPlan& plan);
 
 // What was queued of a run of steps: `steps` of the whole box, and, if torn,
 // some planes further on (a launch failed within a round of slabs).

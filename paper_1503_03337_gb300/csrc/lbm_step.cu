@@ -109,6 +109,8 @@ const char* set_faces(DomainDesc& d, const lbm_geom* g) {
 // not bound by memory in a whole sweep: FP64 by its arithmetic, FP16 and BF16
 // by their issue rate (256^3 D3Q18 FP16: 232 us in whole sweeps, 240 in slabs).
 SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
+  // a boundary pass follows every step: nothing to run several steps of
+  if (d.neq_vel | d.neq_pre) return {};
   if (d.storage != LBM_STORAGE_F32) return {};
   const int64_t plane = (int64_t)d.nx * d.ny * (d.Q * 4 + (d.solid ? 4 : 0));
   if (plane * d.nz * 100 < l2_bytes * 65) return {};
@@ -144,6 +146,26 @@ BlockShape default_block(int Q, int nx, int ny, int64_t N, int storage) {
   int by = 256 / bx;
   while (by > 1 && by / 2 >= ny) by /= 2;
   return {bx, by, 1};
+}
+
+TuneKey tune_key(const DomainDesc& d, const SlabPlan& plan) {
+  return {d.Q, d.storage, d.rounding, d.nx, d.ny, d.nz, d.solid != nullptr, plan.slabs, plan.depth};
+}
+
+bool tune_candidate(const DomainDesc& d, const BlockShape& b) {
+  const int xmax = ((d.nx + 31) / 32) * 32;
+  if (b.bx * b.cpt > xmax && b.bx > 32) return false;
+  // where no step runs two cells per thread
+  if (b.cpt == 2 && (d.storage == LBM_STORAGE_F64 || d.Q == 26 || d.solid ||
+                     wide_offsets(d.Q, d.N)))
+    return false;
+  return true;
+}
+
+int tune_steps(int trials, const SlabPlan& plan) {
+  int unit = plan.slabs > 1 ? plan.depth : 2;
+  unit += unit & 1 ? unit : 0;
+  return (trials + unit - 1) / unit * unit;
 }
 
 cudaError_t launch_step_q14(const DomainDesc& d, int64_t n, int64_t count, BlockShape b,

@@ -1,6 +1,6 @@
 """Launch rules of single-domain steps (csrc/lbm_step.cu): the default block of
-boxes with 64-bit population offsets (CPU), and steps of such a box whose rows
-are not whole warps."""
+boxes with 64-bit population offsets and what the autotuner times (CPU), and
+steps of a wide box whose rows are not whole warps."""
 import os
 import subprocess
 
@@ -36,6 +36,26 @@ def test_wide_boxes_keep_the_row_block(harness, Q, nx, ny, nz, storage):
     assert not linear
     assert bx == min(128, max(32, 1 << (nx - 1).bit_length())) and bx * by == 256
     assert -(-ny // by) <= 65535
+
+
+def test_autotuner_times_what_steps_run(harness):
+    """A choice is shared only by boxes that run the same kernels in the same
+    order; two cells a thread are timed only where a step uses them; boxes
+    with extrapolation faces step in whole sweeps, and slabs are timed in
+    whole rounds with as many even as odd steps."""
+    L2 = 135 << 20
+    cases = [(18, 128, 128, 128, 1) + rest for rest in ((0, 0, 0), (1, 0, 0), (0, 1, 0), (0, 0, 1))]
+    cases += [(18, 64, 64, 64, 2, 0, 0, 0), (18, 64, 64, 64, 2, 1, 0, 0), (14, 280, 280, 64, 1, 0, 0, 0)]
+    got = harness("\n".join("tune %d %d %d %d %d %d %d %d 8 %d" % (c + (L2,)) for c in cases))
+    plans, steps, pairs, keys = ([g[:2] for g in got], [g[2] for g in got], [g[3] for g in got],
+                                 [g[4:] for g in got])
+    assert len(set(keys)) == len(keys)
+    assert plans[0][0] > 1 and plans[1][0] > 1 and plans[2][0] > 1
+    assert plans[3] == plans[4] == plans[5] == (1, 1)
+    for (slabs, depth), n in zip(plans, steps):
+        assert n >= 8 and n % 2 == 0 and (slabs == 1 or n % depth == 0)
+    assert plans[6][0] > 1 and plans[6][1] % 2 == 1
+    assert [p > 0 for p in pairs] == [True, False, True, True, True, False, True]
 
 
 @pytest.mark.gpu
