@@ -178,13 +178,17 @@ class ClockSampler:
 # ---- ncu-derived traffic --------------------------------------------------------
 
 def kernel_source_hash():
-    """Hash of the sources the single-domain step kernel is built from."""
+    """Hash of the sources the single-domain step kernels are built from and
+    their launch order is decided in."""
     h = hashlib.sha256()
     for name in ("lbm_model.cuh", "lbm_factored.cuh", "lbm_collide.cuh", "lbm_kernels.cuh",
-                 "lbm_launch.cuh", "lbm_step.cu", "lbm_step_impl.cuh", "lbm_step_q14.cu",
-                 "lbm_step_q18.cu", "lbm_step_q14h.cu", "lbm_step_q18h.cu", "lbm_step_q14b.cu",
-                 "lbm_step_q18b.cu", "lbm_step_q14sh.cu", "lbm_step_q18sh.cu",
-                 "lbm_step_q14sb.cu", "lbm_step_q18sb.cu"):
+                 "lbm_launch.cuh", "lbm_internal.h", "lbm_step.cu", "lbm_step_impl.cuh",
+                 "lbm_step_q14.cu", "lbm_step_q14b.cu", "lbm_step_q14d.cu", "lbm_step_q14h.cu",
+                 "lbm_step_q14sb.cu", "lbm_step_q14sh.cu",
+                 "lbm_step_q18.cu", "lbm_step_q18b.cu", "lbm_step_q18d.cu", "lbm_step_q18h.cu",
+                 "lbm_step_q18sb.cu", "lbm_step_q18sh.cu",
+                 "lbm_step_q26.cu", "lbm_step_q26b.cu", "lbm_step_q26d.cu", "lbm_step_q26h.cu",
+                 "lbm_step_q26sb.cu", "lbm_step_q26sh.cu"):
         p = os.path.join(ROOT, "paper_1503_03337_gb300", "csrc", name)
         with open(p, "rb") as fh:
             h.update(os.path.basename(p).encode())
@@ -198,7 +202,7 @@ def step_launches(Q, storage, n, updates, l2_bytes):
     rule of slab_plan and run_slabs)."""
     plane = n * n * Q * 4
     touched = min(l2_bytes * 62 // 100 // plane, n)
-    if storage != "f32" or plane * n * 100 < l2_bytes * 65 or touched < (18 if Q == 26 else 10):
+    if storage != "f32" or plane * n * 100 < l2_bytes * 65 or touched < (18 if Q == 26 else 11):
         return updates
     depth = min(16, touched * 3 // 8)
     slabs = -(-(n - depth) // (touched - depth))
@@ -209,8 +213,8 @@ def step_launches(Q, storage, n, updates, l2_bytes):
 
 
 def recorded_traffic(Q, storage, n):
-    """DRAM bytes per launch of the step kernel from the committed ncu summary,
-    if it was taken on the current kernel source (else None)."""
+    """DRAM bytes per update from the committed ncu summary, if it was taken on
+    the current kernel source (else None)."""
     path = os.path.join(ROOT, "profiles", "step_kernel_dram_traffic.txt")
     if not os.path.exists(path):
         return None
@@ -603,7 +607,7 @@ def run_gpu(a, rank, world, dist):
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": traffic, "peak_kind": peak_kind,
-                     "algorithmic_bytes_per_launch": bytes_per_update * cells,
+                     "algorithmic_bytes_per_update": bytes_per_update * cells,
                      "note": "bytes of one update over its time; boxes swept in slabs run "
                              "several updates per trip to memory, so this may exceed the "
                              "copy bandwidth",

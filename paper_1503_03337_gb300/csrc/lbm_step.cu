@@ -101,13 +101,14 @@ const char* set_faces(DomainDesc& d, const lbm_geom* g) {
 // whole sweeps.  A round is 3/8 of the planes a slab touches, at most 16: the
 // round's steps share one trip to memory, but each costs the slab a plane and
 // every launch about 2 us of ramp and tail (128^3: 4 steps 40.4 us, 8 38.1,
-// 16 37.1, 32 37.4).  Fewer than 10 planes (boxes of 350^2 and more) leave
-// little of a round (320^3, with 11, takes 656 us in slabs and 703 whole).  D3Q26 is bound by its registers
-// as much as by memory and wants 18 planes: 160^3 132 us in slabs, 138 in
-// whole sweeps, 208^3 281 and 287, 224^3 375 and 370, 256^3 568 and 536.  The
-// other storage types are
-// not bound by memory in a whole sweep: FP64 by its arithmetic, FP16 and BF16
-// by their issue rate (256^3 D3Q18 FP16: 232 us in whole sweeps, 240 in slabs).
+// 16 37.1, 32 37.4).  Fewer than 11 planes (D3Q18 planes above 320^2) leave
+// rounds of three steps, which run_slabs sweeps whole (320^3, with 11, takes
+// 656 us in slabs and 703 whole).  D3Q26 is bound by its registers as much as
+// by memory and wants 18 planes: 160^3 132 us in slabs, 138 in whole sweeps,
+// 208^3 281 and 287, 224^3 375 and 370, 256^3 568 and 536.  The other storage
+// types are not bound by memory in a whole sweep: FP64 by its arithmetic, FP16
+// and BF16 by their issue rate (256^3 D3Q18 FP16: 232 us in whole sweeps, 240
+// in slabs).
 SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
   // a boundary pass follows every step: nothing to run several steps of
   if (d.neq_vel | d.neq_pre) return {};
@@ -115,7 +116,7 @@ SlabPlan slab_plan(const DomainDesc& d, int64_t l2_bytes) {
   const int64_t plane = (int64_t)d.nx * d.ny * (d.Q * 4 + (d.solid ? 4 : 0));
   if (plane * d.nz * 100 < l2_bytes * 65) return {};
   const int touched = (int)std::min<int64_t>(l2_bytes * 62 / 100 / plane, d.nz);
-  if (touched < (d.Q == 26 ? 18 : 10)) return {};
+  if (touched < (d.Q == 26 ? 18 : 11)) return {};
   SlabPlan p;
   p.depth = std::min(16, touched * 3 / 8);
   const int own = touched - p.depth, share = d.per[2] ? d.nz : d.nz - p.depth;

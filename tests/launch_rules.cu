@@ -3,6 +3,7 @@
 //   block Q nx ny nz storage              ->  bx by linear
 //   tune Q nx ny nz storage solid per_z neq trials l2 -> slabs depth steps, candidates
 //     of two cells a thread, the tuner's key (9 values)
+//   count Q nx ny nz storage updates l2   ->  step launches of a walled box
 #include <cstdio>
 #include <cstring>
 
@@ -30,18 +31,28 @@ int main() {
       std::printf("%d %d %d\n", b.bx, b.by, (int)lbm::steps_in_line(Q, nx, ny, N));
       continue;
     }
-    int solid, trials;
     long long l2;
     lbm::DomainDesc d{};
-    if (std::scanf("%d %d %d %d %lld", &solid, &d.per[2], &d.neq_vel, &trials, &l2) != 5) return 2;
-    const uint32_t mask = 0;  // any address: the rules only ask whether there is one
-    d.solid = solid ? &mask : nullptr;
     d.Q = Q;
     d.nx = nx;
     d.ny = ny;
     d.nz = nz;
     d.N = N;
     d.storage = storage;
+    if (!std::strcmp(what, "count")) {
+      int updates, launches = 0;
+      if (std::scanf("%d %lld", &updates, &l2) != 2) return 2;
+      lbm::run_slabs(nz, false, lbm::slab_plan(d, l2), updates, [&](int64_t, int, int) {
+        ++launches;
+        return cudaSuccess;
+      });
+      std::printf("%d\n", launches);
+      continue;
+    }
+    int solid, trials;
+    if (std::scanf("%d %d %d %d %lld", &solid, &d.per[2], &d.neq_vel, &trials, &l2) != 5) return 2;
+    const uint32_t mask = 0;  // any address: the rules only ask whether there is one
+    d.solid = solid ? &mask : nullptr;
     const lbm::SlabPlan plan = lbm::slab_plan(d, l2);
     int pairs = 0;
     for (int bx : {32, 64, 128}) pairs += lbm::tune_candidate(d, {bx, 1, 2});
