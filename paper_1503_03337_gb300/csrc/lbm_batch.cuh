@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(256, DYN ? 3 : 4)
   pdl_acquire();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane(d);
+  const int z = slab_plane<S>(d);
   if (x >= d.nx || y >= d.ny) return;
   const int x_lo = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   if constexpr (DYN)

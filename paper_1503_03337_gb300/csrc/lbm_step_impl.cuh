@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Dom
   pdl_release();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane(d);
+  const int z = slab_plane<S>(d);
   if (x >= d.nx || y >= d.ny) return;
   // a 32-wide x-range containing x; it is the calling warp's range when
   // blockDim.x is a multiple of 32 (then the path choice is warp-uniform)
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256, 3) k_step_pair(Domain<float> d) {
   pdl_release();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane(d);
+  const int z = slab_plane<S>(d);
   if (x0 >= d.nx || y >= d.ny) return;
   update_pair_even<Q, S, FORCE, SR>(d, static_cast<S*>(d.f), x0 + d.nx * (y + d.ny * z));
 }
@@ -216,10 +216,13 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
     });
     return;
   }
-  // the build of the D3Q18 BF16 stochastic step that carries the solid code is
-  // scheduled better: 244 against 250 us at 256^3 (D3Q14 210 against 200)
-  constexpr bool kSolids = Q == 18 && SR && std::is_same_v<S, __nv_bfloat16>;
+  // The odd D3Q18 BF16 stochastic kernel that carries the solid code is faster
+  // than the one without it: 240.4 against 248.2 us a step at 256^3 (pairs on
+  // even steps), 267.4 against 282.2 one cell a thread; no difference at 128^3.
+  // Registers and spills are the same, the order of instructions is not, and
+  // no other type shares it (D3Q14 210.0 against 197.6, D3Q18 FP16 equal).
   by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
+    constexpr bool kSolids = ODD && Q == 18 && SR && std::is_same_v<S, __nv_bfloat16>;
     launch_one(k_step<Q, S, ODD, FORCE, SR, false, kSolids>, d, grid, block, pdl, st);
   });
 }

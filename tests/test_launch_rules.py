@@ -58,6 +58,16 @@ def test_autotuner_times_what_steps_run(harness):
     assert [p > 0 for p in pairs] == [True, False, True, True, True, False, True]
 
 
+def test_only_fp32_storage_is_swept_in_slabs(harness):
+    """The kernels of the other storage types ignore a launch's first plane."""
+    L2 = 135 << 20
+    got = harness("\n".join("tune %d %d %d 128 %d 0 %d 0 8 %d" % (Q, n, n, storage, per, L2)
+                            for storage in (lbm.LBM_STORAGE_F64, lbm.LBM_STORAGE_F16,
+                                            lbm.LBM_STORAGE_BF16)
+                            for Q in (14, 18, 26) for n in (64, 100, 128, 256) for per in (0, 1)))
+    assert all(g[:2] == (1, 1) for g in got) and len(got) == 72
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("Q,nx,ny,nz", [(18, 33, 70000, 52), (14, 500, 560, 550)])
 def test_wide_box_with_ragged_rows(Q, nx, ny, nz):
