@@ -200,14 +200,14 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2 : 4)
 // loaded values occupy registers for the whole update, so those variants
 // get a looser register cap.  Without DYN the descriptor holds the constant
 // force and the kernel is the single-domain step kernel.
-template <int Q, typename S, bool ODD, bool SR, bool FORCE, bool DYN>
+template <int Q, typename S, bool ODD, bool SR, bool FORCE, bool DYN, bool SLAB>
 __global__ void __launch_bounds__(256, DYN ? 3 : 4)
     k_solo(Domain<float> d, const StepDyn* __restrict__ dyn) {
   pdl_release();
   pdl_acquire();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane<S>(d);
+  const int z = plane_of<SLAB>(d);
   if (x >= d.nx || y >= d.ny) return;
   const int x_lo = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   if constexpr (DYN)
@@ -276,24 +276,24 @@ void launch_group_typed(const GroupLaunch& g) {
     launch_pdl(k_group<Q, S, false, false, FORCE>, g.grid, g.block, true, g.stream, g.ents, g.dyn, g.count, g.tiles, g.per);
 }
 
+template <int Q, typename S, bool SR, bool FORCE, bool DYN>
+void launch_solo_kernel(const SoloLaunch& g) {
+  constexpr bool kSlabs = sizeof(S) == 4;  // only FP32 boxes are swept in slabs
+  const bool slab = kSlabs && is_slab(g.d, (int)g.grid.z);
+  auto kernel = g.odd ? (slab ? k_solo<Q, S, true, SR, FORCE, DYN, kSlabs>
+                              : k_solo<Q, S, true, SR, FORCE, DYN, false>)
+                      : (slab ? k_solo<Q, S, false, SR, FORCE, DYN, kSlabs>
+                              : k_solo<Q, S, false, SR, FORCE, DYN, false>);
+  launch_pdl(kernel, g.grid, g.block, true, g.stream, g.d, g.dyn);
+}
+
 template <int Q, typename S, bool FORCE>
 void launch_solo_typed(const SoloLaunch& g) {
-  if constexpr (Stochastic<S>::enabled) {
-    if (g.sr) {
-      if (g.odd) launch_pdl(k_solo<Q, S, true, true, FORCE, true>, g.grid, g.block, true, g.stream, g.d, g.dyn);
-      else launch_pdl(k_solo<Q, S, false, true, FORCE, true>, g.grid, g.block, true, g.stream, g.d, g.dyn);
-      return;
-    }
-  }
-  if constexpr (FORCE) {
-    if (g.dyn_force) {
-      if (g.odd) launch_pdl(k_solo<Q, S, true, false, true, true>, g.grid, g.block, true, g.stream, g.d, g.dyn);
-      else launch_pdl(k_solo<Q, S, false, false, true, true>, g.grid, g.block, true, g.stream, g.d, g.dyn);
-      return;
-    }
-  }
-  if (g.odd) launch_pdl(k_solo<Q, S, true, false, FORCE, false>, g.grid, g.block, true, g.stream, g.d, g.dyn);
-  else launch_pdl(k_solo<Q, S, false, false, FORCE, false>, g.grid, g.block, true, g.stream, g.d, g.dyn);
+  if constexpr (Stochastic<S>::enabled)
+    if (g.sr) return launch_solo_kernel<Q, S, true, FORCE, true>(g);
+  if constexpr (FORCE)
+    if (g.dyn_force) return launch_solo_kernel<Q, S, false, true, true>(g);
+  launch_solo_kernel<Q, S, false, FORCE, false>(g);
 }
 
 template <int Q, typename L, template <int, typename, bool> class Op>

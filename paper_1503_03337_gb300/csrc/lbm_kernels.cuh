@@ -130,20 +130,26 @@ __host__ __device__ inline void fill_offsets(Domain<R>& d) {
   }(std::make_integer_sequence<int, Q>{});
 }
 
-// Plane of the calling CTA in a launch of gridDim.z planes from d.z0 on; past
-// the last plane it goes on at plane 0 (slabs of a box periodic in z).  Only
-// FP32 storage is swept in slabs (slab_plan); the others take the plane from
-// the grid alone: their steps are bound by issue and the extra operations cost
-// up to 2 % (D3Q18 stochastic BF16, us a step with and without: 256^3 244.6
-// and 238.9, 128^3 28.9 and 28.4).
-template <typename S, typename R>
-__device__ __forceinline__ int slab_plane(const Domain<R>& d) {
-  if constexpr (sizeof(S) == 4) {
+// Plane of the calling CTA.  SLAB: the launch covers gridDim.z planes from d.z0
+// on, and past the last plane goes on at plane 0 (slabs of a box periodic in
+// z).  Launches over the whole box have kernels of their own, because these
+// two operations change the schedule of the whole update: us a step in whole
+// sweeps with and without them, D3Q14 FP32 256^3 311.6 and 292.3, 128^3 39.5
+// and 37.7; D3Q18 stochastic BF16 256^3 244.6 and 238.9; D3Q18 FP32 unchanged.
+template <bool SLAB, typename R>
+__device__ __forceinline__ int plane_of(const Domain<R>& d) {
+  if constexpr (SLAB) {
     const int z = d.z0 + (int)blockIdx.z;
     return z < d.nz ? z : z - d.nz;
   } else {
     return (int)blockIdx.z;
   }
+}
+
+// Does a launch over `planes` planes from d.z0 on need a SLAB kernel?
+template <typename R>
+inline bool is_slab(const Domain<R>& d, int planes) {
+  return d.z0 != 0 || planes != d.nz;
 }
 
 // Edge-profile factor of moving face `face` for a cell whose position bits

@@ -36,13 +36,13 @@ constexpr int step_min_blocks() {
 // a trigger before it makes several later grids resident, whose blocks take
 // whatever slots are free and bunch on some SMs (33^3 D3Q14 FP32: 3.07 us a
 // step with the trigger first, 2.87 so; boxes of many waves do not change).
-template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool WIDE, bool SOLIDS>
+template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool WIDE, bool SOLIDS, bool SLAB>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Domain<float> d) {
   pdl_acquire();
   pdl_release();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane<S>(d);
+  const int z = plane_of<SLAB>(d);
   if (x >= d.nx || y >= d.ny) return;
   // a 32-wide x-range containing x; it is the calling warp's range when
   // blockDim.x is a multiple of 32 (then the path choice is warp-uniform)
@@ -133,13 +133,13 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(
 // thread to local memory, and is still faster than at two blocks without
 // spills (measured at 256^3: FP16 66.4 vs 62.7 GLUPS for Q18, 85.0 vs 81.7
 // for Q14).
-template <int Q, typename S, bool FORCE, bool SR>
+template <int Q, typename S, bool FORCE, bool SR, bool SLAB>
 __global__ void __launch_bounds__(256, 3) k_step_pair(Domain<float> d) {
   pdl_acquire();
   pdl_release();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = slab_plane<S>(d);
+  const int z = plane_of<SLAB>(d);
   if (x0 >= d.nx || y >= d.ny) return;
   update_pair_even<Q, S, FORCE, SR>(d, static_cast<S*>(d.f), x0 + d.nx * (y + d.ny * z));
 }
@@ -185,10 +185,15 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
   const dim3 block(b.bx, b.by);
   const int by = (d.ny + b.by - 1) / b.by;
   const dim3 grid((d.nx + b.bx - 1) / b.bx, by, planes);
+  // only FP32 boxes are swept in slabs (slab_plan)
+  constexpr bool kSlabs = sizeof(S) == 4;
+  const bool slab = kSlabs && is_slab(d, planes);
   // Q*N >= 2^31: one cell per thread with 64-bit population offsets
   if (wide) {
     by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
-      launch_one(k_step<Q, S, ODD, FORCE, SR, true, true>, d, grid, block, pdl, st);
+      launch_one(slab ? k_step<Q, S, ODD, FORCE, SR, true, true, kSlabs>
+                      : k_step<Q, S, ODD, FORCE, SR, true, true, false>,
+                 d, grid, block, pdl, st);
     });
     return;
   }
@@ -199,8 +204,10 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
   if constexpr (Q != 26) {
     if (b.cpt == 2 && !odd && d.nx % 2 == 0 && !d.solid) {
       const dim3 half((d.nx / 2 + b.bx - 1) / b.bx, by, planes);
-      if (force) launch_one(k_step_pair<Q, S, true, SR>, d, half, block, pdl, st);
-      else launch_one(k_step_pair<Q, S, false, SR>, d, half, block, pdl, st);
+      by_flags(false, force, [&]<bool ODD, bool FORCE>() {
+        launch_one(slab ? k_step_pair<Q, S, FORCE, SR, kSlabs> : k_step_pair<Q, S, FORCE, SR, false>,
+                   d, half, block, pdl, st);
+      });
       return;
     }
   }
@@ -223,7 +230,9 @@ void launch_parity(const Domain<float>& d, bool odd, bool force, bool wide, int 
   // no other type shares it (D3Q14 210.0 against 197.6, D3Q18 FP16 equal).
   by_flags(odd, force, [&]<bool ODD, bool FORCE>() {
     constexpr bool kSolids = ODD && Q == 18 && SR && std::is_same_v<S, __nv_bfloat16>;
-    launch_one(k_step<Q, S, ODD, FORCE, SR, false, kSolids>, d, grid, block, pdl, st);
+    launch_one(slab ? k_step<Q, S, ODD, FORCE, SR, false, kSolids, kSlabs>
+                    : k_step<Q, S, ODD, FORCE, SR, false, kSolids, false>,
+               d, grid, block, pdl, st);
   });
 }
 
