@@ -303,8 +303,13 @@ int lbm_residual(lbm_handle *h, int32_t kind, int32_t component, double *r);
  * multiply-adds differently than in the one-cell kernel, so results agree to
  * FP32 rounding, not bit for bit. */
 typedef struct lbm_launch {
-  int32_t bx, by;           /* threads along x (multiple of 32, so a warp never
-                               spans two x-rows) and y; bx*by <= 256          */
+  int32_t bx, by;           /* threads along x (multiple of 32) and y; bx*by <=
+                               256.  Steps by rows: a warp never spans two
+                               x-rows.  Steps in linear order (FP64 storage,
+                               solid nodes, and boxes of 100 thousand cells or
+                               more whose nx is not a multiple of 32) run the
+                               cells one after another whatever row they are
+                               in: only bx*by matters there.                  */
   int32_t cells_per_thread; /* 1, or 2: on even steps with nx even, each
                                thread updates the x-adjacent cells 2t, 2t+1,
                                moving each population of the pair as one

@@ -46,7 +46,7 @@ struct FieldArgs {
 // by the zeros of c.  p_ref enters P as one constant, sum_a 3 w_a p_ref =
 // 3 (1 - w0) p_ref.  160^3 D3Q18 FP32: writing populations takes 145 us and
 // reading them 290 (0.89 GB either way), u and p 638, initialising 583;
-// restoring, reducing, reading u and p and ten steps took 2.69 ms, 2.03 now.
+// restoring, reducing, reading u and p and ten steps took 2.69 ms, 1.88 now.
 
 // Cells i of a grid-stride loop over 32-bit indices (N < 2^31).
 template <typename Fn>
@@ -152,17 +152,14 @@ struct ReduceArgs {
   double edge_scale[6][2];  // their edge profiles (Domain::edge_scale)
 };
 
-// Blocks of a reduction: four resident ones per SM, each looping over cells,
-// so that the FP64 end of a block is paid four times an SM.
-constexpr int kReduceGrid = 608;
-static_assert(kReduceGrid <= kReduceBlocks, "partials buffer");
-
 // The block's statistics from every thread's v, to partials[k * gridDim.x +
 // blockIdx.x].  FP64 adds run at two lanes per clock and SM, so their number
 // is what this costs: the threads' values are laid out in shared memory and
 // one warp sums statistic k, 32 lanes of a few values each and five shuffles
 // (180 warp adds a block of 256 threads; reducing all fifteen by shuffles in
-// every warp took 700 and 5 us a block, on eight blocks an SM).
+// every warp took 700 and 5 us a block).  A reduction runs four resident blocks
+// per SM (kReduceBlocks), each looping over cells, so it is paid four times an
+// SM; eight times before.
 __device__ __forceinline__ void block_partials(const double (&v)[kNumStats], double* partials) {
   __shared__ double shm[kNumStats][kReduceThreads];
 #pragma unroll
@@ -517,7 +514,7 @@ cudaError_t launch_reduce(const DomainDesc& dd, int64_t n, double* u_prev, int h
     for (int k = 0; k < 2; ++k) a.edge_scale[face][k] = dd.edge_scale[face][k];
   }
   int64_t g = (dd.N + kReduceThreads - 1) / kReduceThreads;
-  if (g > kReduceGrid) g = kReduceGrid;
+  if (g > kReduceBlocks) g = kReduceBlocks;
   if (g < 1) g = 1;
   const bool odd = n & 1;
   const Domain<float> df = to_domain<float>(dd, F);

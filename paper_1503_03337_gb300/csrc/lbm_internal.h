@@ -15,7 +15,7 @@ namespace lbm {
 // the two step counters): 3 du, 3 u, 3 u_prev, P, 3 flux, max, nonfinite.
 constexpr int kNumSums = 14;   // summed entries
 constexpr int kNumStats = 15;  // plus the max
-constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs; partials per reduction
+constexpr int kReduceBlocks = 608;  // at most, of a reduction: 4 x 152 SMs
 constexpr int kReduceThreads = 256;
 
 // Everything a kernel needs to know about one domain, in FP64; the launchers

@@ -544,17 +544,10 @@ __host__ __device__ __forceinline__ bool warp_any(bool v) {
 #endif
 }
 
-// The whole fused update of one cell: gather (stream), collide, scatter.
-// Odd steps pick one of three addressing variants.  `x_lo`..`x_hi` is the
-// x-range of the calling warp: when a warp lies within one x-row (block
-// width a multiple of 32) every test below is uniform across the warp, so
-// the variants never diverge inside a warp.  The two boundary variants come
-// with and without the mirrored links of symmetry faces (d.sym is uniform
-// across the grid), so domains without one pay nothing for them.
-// update_cell_at reads the step's body force F[0..2] and rounding key *key
-// where they are used (F and key may live outside the descriptor);
-// update_cell takes them from the descriptor.  SOLIDS = false: the domain has
-// no solid mask (batched domains).
+// The whole fused update of one cell: gather (stream), collide, scatter, with
+// the step's body force F[0..2] and rounding key *key, which are read where
+// they are used and may live outside the descriptor.  SOLIDS = false: the
+// caller's domains have no solid mask.
 
 // Even step of cell i: its own slots only.
 template <int Q, typename S, typename R, bool FORCE, bool SR, bool CG, bool WIDE, bool SOLIDS>
@@ -566,7 +559,11 @@ __host__ __device__ __forceinline__ void update_even(const Domain<R>& d, S* __re
 }
 
 // Odd step of cell i = (x, y, z); bulk_yz: no cell of the warp lies on a y or
-// z face, bulk_x: none at a row end (both uniform across the warp).
+// z face, bulk_x: none at a row end.  Both are uniform across the warp, so it
+// runs one addressing variant: tabled offsets in the bulk, x-only beside row
+// ends, or the full one, the last two with or without the mirrored links of
+// symmetry faces (d.sym is uniform across the grid); four more, with the
+// cells' solid bits, where a link of the warp touches a solid node.
 template <int Q, typename S, typename R, bool FORCE, bool SR, bool CG, bool WIDE, bool SOLIDS>
 __host__ __device__ __forceinline__ void update_odd(const Domain<R>& d, S* __restrict__ f,
                                                     const R* F, const uint32_t* key, int i, int x,
@@ -621,6 +618,9 @@ __host__ __device__ __forceinline__ void update_odd(const Domain<R>& d, S* __res
   }
 }
 
+// Step of cell (x, y, z) of a launch by rows.  `x_lo`..`x_hi` is the x-range of
+// the calling warp, which lies within one x-row (block width a multiple of
+// 32), so the choice of variant is uniform across it.
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,
           bool CG = false, bool WIDE = false, bool SOLIDS = true>
 __host__ __device__ __forceinline__ void update_cell_at(const Domain<R>& d, S* __restrict__ f,
@@ -635,6 +635,7 @@ __host__ __device__ __forceinline__ void update_cell_at(const Domain<R>& d, S* _
         x_lo > 0 && x_hi < d.nx - 1);
 }
 
+// update_cell_at with the force and key of the descriptor.
 template <int Q, typename S, typename R, bool ODD, bool FORCE, bool SR = false,
           bool CG = false, bool WIDE = false, bool SOLIDS = true>
 __host__ __device__ __forceinline__ void update_cell(const Domain<R>& d, S* __restrict__ f,

@@ -62,12 +62,15 @@ struct LineArgs {
 // no lanes are left empty at the ends of rows; the warp votes on the
 // addressing variant.  The step is bound by instruction issue in L2-sized
 // boxes and with 2-byte storage, so what it gains is the padding: us a step by
-// rows and so, 97x97x49 D3Q18 FP32 10.8 and 9.6, 65^3 8.4 and 6.8, 129^3 47.2
+// rows and so, lid-driven boxes with walls on every other face, 97x97x49 D3Q18
+// FP32 10.8 and 9.6 (11.5 and 10.7 with a symmetry plane on a z face, whose
+// mirrored addressing every row end then takes), 65^3 8.4 and 6.8, 129^3 47.2
 // and 41.8, 200^3 154 and 146, 97^3 FP16 17.2 and 13.6, 161^3 FP16 75.9 and
 // 67.4, 100^3 D3Q26 FP16 34.8 and 23.9.  The coordinates of a cell are formed
 // before the wait for the previous step.  SOLIDS: d has a solid mask; every
-// such box runs here (100^3, 30 % solid, FP32: 20.9 and 17.8; 192^3, whose rows
-// have no padding, 137.7 and 137.0), so k_step carries no solid code.
+// such box without 64-bit offsets runs here (100^3, 30 % solid, FP32: 20.9 and
+// 17.8; 192^3, whose rows have no padding, 137.7 and 137.0), so of k_step's
+// builds only those with 64-bit offsets need the solid code.
 template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool SOLIDS>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, S>()) k_step_line(Domain<float> d,
                                                                             LineArgs a) {
