@@ -101,12 +101,15 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S>()) k_step_line(Doma
 // rows half of it, 65-wide ones a third), as does any branch that splits a
 // warp, so every cell takes the general addressing.  Launched with one warp
 // per block (default_block): the warps then spread evenly over the SMs.
-// 16x16x32 D3Q18: 30.8 us a step with 32 x 8 blocks of rows, 8.2 so.
+// 16x16x32 D3Q18: 28.5 us a step with 32 x 8 blocks of rows, 8.0 so.
 template <int Q, bool ODD, bool FORCE, bool WIDE>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(Domain<double> d) {
-  // before the wait: with so many small blocks a late trigger costs more than
-  // the even spread gains (16x16x32 D3Q18: 8.2 us a step so, 9.2 after it)
-  pdl_release();
+  // No trigger: the next launch comes in as the blocks of this one end.  Blocks
+  // that are let in earlier take whatever slots free first, so that some SMs
+  // hold more of them than others, and an SM's time goes by its warps (us a
+  // step with the trigger before the wait, after it and without: D3Q18
+  // 16x16x32 8.3, 8.2, 8.0; 32^3 32.6, 14.8, 14.7; 256x256x1 38.2, 38.2, 28.5;
+  // D3Q26 31^3 44.8, 44.7, 27.6; 64^3 and more the same).
   pdl_acquire();
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // N < 2^31
   if (t >= (unsigned)d.N) return;
