@@ -82,6 +82,18 @@ const char* set_faces(DomainDesc& d, const lbm_geom* g);
 cudaError_t launch_solid_links(const DomainDesc& d, const uint8_t* bytes, uint32_t* links,
                                cudaStream_t st);
 
+// Do d's step and boundary launches let the next one in only as their blocks
+// end?  Blocks of a boundary pass that is let in early take the first slots
+// that free as the step drains, bunch on a few SMs, and the nodes of x faces (a
+// line of memory per lane) then take long.  us a step, let in early and held
+// back: D3Q14 FP32 64^3 14.5 and 9.9, 128^3 with x faces 57.0 and 43.7; D3Q18
+// FP16 64^3 21.1 and 12.7, 28^3 8.3 and 8.0.  In smaller boxes it costs more
+// than it gains (D3Q26 FP32 12^3 8.1 and 8.8, D3Q18 FP32 20^3 6.2 and 6.5),
+// except with FP64 storage, whose steps let nothing in early (k_step_f64).
+inline bool holds_next(const DomainDesc& d) {
+  return (d.neq_vel | d.neq_pre) && (d.storage == LBM_STORAGE_F64 || d.N >= 16384);
+}
+
 // Non-equilibrium extrapolation of the boundary nodes of d's LBM_NEQ_*
 // faces, on the populations of step n (after the step n-1 -> n).
 cudaError_t launch_neq(const DomainDesc& d, int64_t n, bool pdl, cudaStream_t st);

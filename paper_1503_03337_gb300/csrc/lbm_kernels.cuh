@@ -40,6 +40,7 @@ struct Domain {
   Rates<R> s;
   R F[3];            // body force at the step's time level t_n
   uint32_t key;      // per-step key of the stochastic-rounding hash
+  int hold;          // the next launch comes in only as the blocks of this one end
   // Solid nodes (general geometry), null if none: per cell, bit a set if
   // the pull source x - c_a (after periodic wraps and symmetry mirrors; not
   // beyond a wall) is a solid node, so that link bounces back off a wall at

@@ -31,12 +31,13 @@ namespace {
 // storage the two FP64 lanes of an SM bound it.  One or two warps a block
 // spread the nodes over all SMs (65x33x33 D3Q14 FP64, 14 thousand nodes: 223
 // or 446 blocks instead of 56; with the shorter arithmetic a step of that box
-// takes 42.8 us instead of 44.4).
+// took 42.8 us instead of 44.4; 26.6
+// since its steps let nothing in early).
 constexpr int kNeqThreads = 64;
 
 template <int Q, typename S, typename R, bool ODD>
 __global__ void __launch_bounds__(kNeqThreads) k_neq(Domain<R> d, NeqArgs a) {
-  pdl_release();
+  if (!d.hold) pdl_release();
   pdl_acquire();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < a.off[6]) neq_node<Q, S, R, ODD>(d, a, t);
@@ -47,7 +48,8 @@ void launch_typed(const DomainDesc& dd, int64_t n, const NeqArgs& a, bool pdl,
                   cudaStream_t st) {
   double F[3];
   force_at(dd, n, F);
-  const Domain<R> d = to_domain<R>(dd, F);
+  Domain<R> d = to_domain<R>(dd, F);
+  d.hold = holds_next(dd);
   const int threads = sizeof(R) == 8 ? 32 : kNeqThreads;
   const int blocks = (a.off[6] + threads - 1) / threads;
   launch_pdl((n & 1) ? k_neq<Q, S, R, true> : k_neq<Q, S, R, false>, dim3(blocks), dim3(threads),

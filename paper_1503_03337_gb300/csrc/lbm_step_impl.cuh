@@ -36,10 +36,11 @@ constexpr int step_min_blocks() {
 // a trigger before it makes several later grids resident, whose blocks take
 // whatever slots are free and bunch on some SMs (33^3 D3Q14 FP32: 3.07 us a
 // step with the trigger first, 2.87 so; boxes of many waves do not change).
+// Boxes with extrapolation faces hold it back (holds_next).
 template <int Q, typename S, bool ODD, bool FORCE, bool SR, bool WIDE, bool SOLIDS, bool SLAB>
 __global__ void __launch_bounds__(256, step_min_blocks<Q, S, WIDE>()) k_step(Domain<float> d) {
   pdl_acquire();
-  pdl_release();
+  if (!d.hold) pdl_release();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = plane_of<SLAB>(d);
@@ -81,14 +82,14 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, S>()) k_step_line(Doma
   S* const f = static_cast<S*>(d.f);
   if constexpr (!ODD) {
     pdl_acquire();
-    pdl_release();
+    if (!d.hold) pdl_release();
     update_even<Q, S, float, FORCE, SR, false, false, SOLIDS>(d, f, d.F, &d.key, i);
   } else {
     const int r = a.by_x(i), z = a.by_y(r), x = i - r * d.nx, y = r - z * d.ny;
     const bool yz = y == 0 || y == d.ny - 1 || z == 0 || z == d.nz - 1;
     const bool bulk_yz = !warp_any(yz), bulk_x = !warp_any(x == 0 || x == d.nx - 1);
     pdl_acquire();
-    pdl_release();
+    if (!d.hold) pdl_release();
     update_odd<Q, S, float, FORCE, SR, false, false, SOLIDS>(d, f, d.F, &d.key, i, x, y, z,
                                                              bulk_yz, bulk_x);
   }
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<Q, double>()) k_step_f64(
 template <int Q, typename S, bool FORCE, bool SR, bool SLAB>
 __global__ void __launch_bounds__(256, 3) k_step_pair(Domain<float> d) {
   pdl_acquire();
-  pdl_release();
+  if (!d.hold) pdl_release();
   const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = plane_of<SLAB>(d);
@@ -256,6 +257,7 @@ cudaError_t launch_typed(const DomainDesc& dd, int64_t n, int64_t count, BlockSh
   const bool force = dd.force[0] != 0.0 || dd.force[1] != 0.0 || dd.force[2] != 0.0;
   Domain<R> d = to_domain<R>(dd, zero);
   const bool wide = wide_offsets(dd.Q, dd.N);
+  d.hold = holds_next(dd);
   return run_slabs(dd.nz, dd.per[2] != 0, plan, count, [&](int64_t s, int z0, int planes) {
     double F[3];
     force_at(dd, n + s, F);
