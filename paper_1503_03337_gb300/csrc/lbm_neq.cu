@@ -31,8 +31,8 @@ namespace {
 // storage the two FP64 lanes of an SM bound it.  One or two warps a block
 // spread the nodes over all SMs (65x33x33 D3Q14 FP64, 14 thousand nodes: 223
 // or 446 blocks instead of 56; with the shorter arithmetic a step of that box
-// took 42.8 us instead of 44.4; 26.6
-// since its steps let nothing in early).
+// took 42.8 us instead of 44.4, and takes 26.6 since its steps let nothing in
+// early).
 constexpr int kNeqThreads = 64;
 
 template <int Q, typename S, typename R, bool ODD>
